@@ -52,6 +52,7 @@ __device__ __forceinline__ void store_X(const Dev& D, size_t e, float X) {
 
 __global__ void k_init_state(Dev D) {
     size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (D.t0 && e == 0) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(*D.t0));
     if (e >= (size_t)D.M * D.Npad) return;
     int a = int(e / D.Npad), p = int(e % D.Npad);
     float rho = rho_val(D.rho_idx[a]);

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "acct_admm.h"
 #include "block_admm.h"
 #include "polish.h"
 #include "solver.h"
@@ -391,6 +392,70 @@ static double ms_between(cudaEvent_t a, cudaEvent_t b) {
 }
 
 // ---------------------------------------------------------------------------
+// the account-resident iterations: which books take them, in which launches
+// ---------------------------------------------------------------------------
+struct AcctClass {
+    int first, count;                   // its accounts in the order list (all of them when not ragged)
+    AcctShape shape;
+};
+
+// Time of one iteration of the whole book, us, as measured at 500 to 10,000 assets, 16 to 64 factors and
+// 16 to 500 accounts. Account-resident: 4.5 for the chain of reductions, 2.5 more when it crosses a
+// cluster, and the products with the CTA's rows; times the waves of clusters.
+static double acct_iteration_us(const AcctShape& s, int n, int M, int K, int bytes, int sms) {
+    const int regs = s.threads > 256 ? 128 : 232;
+    const int per_sm = std::max(1, std::min((int)(228 * 1024 / (s.smem + 1024)), 65536 / (s.threads * regs)));
+    const double at_once = std::max(1.0, (s.cluster > 4 ? 0.85 : 1.0) * sms * per_sm / s.cluster);
+    const double one = 4.5 + (s.cluster > 1 ? 2.5 : 0.0) + (bytes > 2 ? 6e-5 : 5e-5) * cdiv(n, s.cluster) * K;
+    return std::ceil(M / at_once) * one * (per_sm > 1 ? 1.3 : 1.0);
+}
+// Batched: the latency of its launches (with the iterations that a chunk runs past the last account's)
+// and the traffic; books with tax lots, tilts, caps or factor bounds take the staged prox on every call.
+static double batched_iteration_us(int M, int N, bool bf16, bool staged) {
+    return (staged ? 60.0 : 30.0) + (bf16 ? 9e-6 : 3e-5) * M * N;
+}
+
+static bool acct_route(const prism_solve_opts& o, bool plain, bool fp64, bool bf16, bool ragged, int M, int N, int K,
+                       bool pw, bool fac, bool cap, const std::vector<int64_t>& offs, std::vector<AcctClass>& classes,
+                       std::vector<int>& order) {
+    // an option that names a form of the batched kernels keeps the book on them, and so does the
+    // failure-path test of their tensor-core waits
+    if (o.fold_products || o.xupdate_form || o.chains || o.g2_sets || !o.fuse_prox || o.ragged_layout == 1) return false;
+    if (std::getenv("PRISM_TEST_STALLED_WAIT_NS")) return false;
+    const int bytes = fp64 ? 8 : (bf16 ? 2 : 4);
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(1, sms);
+    classes.clear();
+    order.clear();
+    double us = 0.0;
+    if (!ragged) {
+        classes.push_back({0, M, acct_shape(N, K, bytes, fp64, fac, pw)});
+        if (classes[0].shape.E == 0) return false;
+        us = acct_iteration_us(classes[0].shape, N, M, K, bytes, sms);
+    } else {
+        // accounts largest first; a class ends where half the entries would do, so that small accounts
+        // take small blocks, several to an SM
+        order.resize(M);
+        for (int a = 0; a < M; ++a) order[a] = a;
+        auto size = [&](int a) { return (int)(offs[a + 1] - offs[a]); };
+        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return size(x) > size(y); });
+        for (int i = 0; i < M;) {
+            const int n = size(order[i]);
+            AcctClass c{i, 0, acct_shape(n, K, bytes, true, fac, pw)};
+            if (c.shape.E == 0) return false;
+            while (i < M && (size(order[i]) > n / 2 || n <= 128)) { ++c.count; ++i; }
+            us += acct_iteration_us(c.shape, n, c.count, K, bytes, sms);
+            classes.push_back(c);
+        }
+    }
+    // single accounts and the packed layout have no batched form
+    if (plain || o.ragged_layout == 2) return true;
+    return us <= batched_iteration_us(M, N, bf16, pw || cap || fac);
+}
+
+// ---------------------------------------------------------------------------
 // one batched solve (all accounts share the launch sequence)
 // ---------------------------------------------------------------------------
 static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solve_opts* o,
@@ -545,6 +610,13 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     if (b->asset_idx && !plain) {
         packed = o->ragged_layout == 2;
     }
+    // ---- which iterations: account-resident (acct_admm.cuh) where its accounts fit and it is the faster
+    std::vector<AcctClass> classes;
+    std::vector<int> order_h;
+    const bool acct = acct_route(*o, plain, fp64, batched_mode_bf16, b->asset_idx != nullptr, M, N, K, has_pw, has_fac_in,
+                                 b->turnover_cap != nullptr, offs, classes, order_h);
+    if (acct) packed = false;
+    const bool lists = packed || (acct && b->asset_idx);   // per-account position lists are needed
     // ---- workspace layout
     const size_t MN = (size_t)M * Npad;
     int tc_chunk = 0;
@@ -553,6 +625,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     int* dsel = nullptr;               // device copy of SC.hsel (polish batches)
     BlkArgs<double> P64;               // PLAIN_FP64: the FP64 per-account kernel's arguments
     BlkArgs<float> PK;                 // ragged books, packed layout: the FP32 per-account kernel's
+    unsigned long long* t0_dev = nullptr;   // device clock at the start of the solve
     auto layout = [&](Arena& A, Dev& D, PolDev& P, BatchDev& BD, void** stage, int** member, int** err,
                       int** pwidx_dev, double** ragged_out) {
         BD.w0 = A.take<double>(MN); BD.lo = A.take<double>(MN); BD.up = A.take<double>(MN); BD.c = A.take<double>(MN);
@@ -627,8 +700,9 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         // packed layout of a ragged book: position lists, sector ranges, processing order, FP32
         // state and input copies for accounts too large for shared memory
         const size_t np = packed ? (size_t)nnz : 0;
-        PK.plist = A.take<int>(np); PK.psec = A.take<int>(packed ? (size_t)M * (S + 1) : 0);
-        PK.order = A.take<int>(packed ? M : 0); PK.queue = A.take<int>(4);
+        PK.plist = A.take<int>(lists ? (size_t)nnz : 0); PK.psec = A.take<int>(lists ? (size_t)M * (S + 1) : 0);
+        PK.order = A.take<int>(lists ? M : 0); PK.queue = A.take<int>(4);
+        t0_dev = A.take<unsigned long long>(1);
         PK.z = A.take<float>(np); PK.y = A.take<float>(np); PK.X = A.take<float>(np);
         PK.w0p = A.take<float>(np); PK.lop = A.take<float>(np); PK.upp = A.take<float>(np); PK.cp = A.take<float>(np);
         PK.pwp = A.take<int>(np);
@@ -842,7 +916,8 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     } else {
         D.s = nullptr; D.ys = nullptr; D.sflag = nullptr; D.rps = nullptr; D.rds = nullptr;
     }
-    D.stream_prox = (pwidx == nullptr && !BD.has_cap) ? 1 : 0;
+    D.stream_prox = (!acct && pwidx == nullptr && !BD.has_cap) ? 1 : 0;
+    D.t0 = t0_dev;
     // the streaming pass runs inside the tensor-core x-update when the roots kernel can hold
     // the account's candidate masks
     D.fused = (D.stream_prox && batched_mode_bf16 && U.nq <= XP_NQMAX && o->fuse_prox) ? 1 : 0;
@@ -883,7 +958,6 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         P64.alpha = o->alpha; P64.eps = o->eps_admm; P64.rho0 = o->rho0;
         P64.max_iter = o->max_iter; P64.min_iter = o->min_iter; P64.adapt_every = D.adapt_every;
     }
-    std::vector<int> order_h;
     if (packed) {
         PK.M = M; PK.N = N; PK.Npad = Npad; PK.K = K; PK.S = S;
         PK.B = U.d_B32; PK.Bp = U.d_B32p; PK.f = U.d_f32; PK.d = U.d_d32; PK.mu = U.d_mu32;
@@ -911,6 +985,8 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         PK.stage_cap = (int)std::min<int64_t>(nmax, (int64_t)(room / per));
         PRISM_CUDA_TRY(cudaMemcpyAsync(PK.order, order_h.data(), (size_t)M * 4, cudaMemcpyHostToDevice, st));
     }
+    if (acct && b->asset_idx)
+        PRISM_CUDA_TRY(cudaMemcpyAsync(PK.order, order_h.data(), (size_t)M * 4, cudaMemcpyHostToDevice, st));
     // ---- control init
     {
         int j0 = (int)std::lround(RHO_PER_DECADE * std::log10(std::max(o->rho0, 1e-12) / RHO_MIN));
@@ -1113,9 +1189,75 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     };
     // the first iterations run the staged prox: the streaming form needs the budget multiplier
     // to have settled (its moves set the streaming form's margin) to keep its candidate lists short
-    const bool blockwise = fp64 || packed;         // every iteration inside the per-account kernel
+    const bool blockwise = acct || fp64 || packed;   // every iteration inside a per-account kernel
     const int cold = (D.stream_prox && !blockwise) ? std::min(std::max(0, o->stream_after), o->max_iter) : 0;
-    if (fp64) {
+    AcctArgs<float> AF;
+    AcctArgs<double> AD;
+    if (acct) {
+        auto fill = [&](auto& A) {
+            A.M = M; A.N = N; A.Npad = Npad; A.K = K; A.S = S;
+            A.sec_start = U.d_sec_start;
+            A.pw_idx = pwidx; A.pw_nbp = BD.pw_nbp;
+            A.nu = D.nu; A.eta_hi = D.eta_hi; A.eta_lo = D.eta_lo; A.theta = D.theta; A.zf = D.z;
+            A.rho_idx = D.rho_idx; A.iters = D.iters; A.active = D.active; A.status = D.status;
+            if (b->asset_idx) { A.plist = PK.plist; A.poff = PA.offsets; A.psec = PK.psec; }
+            if (BD.has_fac) A.sflag = D.sflag;
+            A.t0 = t0_dev;
+            A.alpha = o->alpha; A.eps = o->eps_admm;
+            A.max_iter = o->max_iter; A.min_iter = o->min_iter; A.adapt_every = D.adapt_every;
+        };
+        fill(AF);
+        fill(AD);
+        if (batched_mode_bf16) AF.B16p = U.d_B16p; else AF.B32p = U.d_B32p;
+        AF.f = U.d_f32; AF.d = U.d_d32; AF.mu = U.d_mu32;
+        if (!b->asset_idx) { AF.Cinv = D.Cinv; AF.G = D.G; }   // (of the split-off factor block when there is one)
+        AF.w0 = BD.w0f; AF.lo = BD.lof; AF.up = BD.upf; AF.c = BD.cf;
+        AF.pw_bp = BD.pw_bpf; AF.pw_sl = BD.pw_slf;
+        AF.band_lo = BD.band_lof; AF.band_hi = BD.band_hif;
+        AF.z = D.z; AF.y = D.y;
+        if (BD.has_cap) AF.tau = BD.tauf;
+        if (BD.has_fac) { AF.flo = BD.flof; AF.fhi = BD.fhif; AF.s = D.s; AF.ys = D.ys; }
+        AD.B64 = U.d_B64; AD.f = U.d_f64; AD.d = U.d_d64; AD.mu = U.d_mu64;
+        AD.w0 = BD.w0; AD.lo = BD.lo; AD.up = BD.up; AD.c = BD.c;
+        AD.pw_bp = BD.pw_bp; AD.pw_sl = BD.pw_sl;
+        AD.band_lo = BD.band_lo; AD.band_hi = BD.band_hi;
+        AD.z = P64.z; AD.y = P64.y;
+        if (BD.has_cap) AD.tau = BD.tau;
+        if (BD.has_fac) { AD.flo = BD.flo; AD.fhi = BD.fhi; AD.s = P64.s_state; AD.ys = P64.ys_state; }
+    }
+    // the accounts' iterations, one launch per class of sizes (side by side on the chains' streams)
+    auto run_acct = [&](int resume, double eps, int max_iter) {
+        if (o->time_budget_s > 0) {
+            const double left = o->time_budget_s - std::chrono::duration<double>(std::chrono::steady_clock::now() - t_call0).count();
+            AF.budget_ns = AD.budget_ns = (unsigned long long)(std::min(std::max(left, 0.0), 1e9) * 1e9) + 1;
+        }
+        AF.resume = AD.resume = resume;
+        AF.eps = (float)eps; AD.eps = eps;
+        AF.max_iter = AD.max_iter = max_iter;
+        const int nstream = SC.chains_ok && !SC.prof.on ? std::min<int>(SolveCache::MAXCH, (int)classes.size()) : 1;
+        SC.prof.run(PRISM_K_BLOCK, (int)classes.size(), st, [&] {
+            if (nstream > 1) cudaEventRecord(SC.ev_fork, st);
+            for (int c = 1; c < nstream; ++c) cudaStreamWaitEvent(SC.chst[c - 1], SC.ev_fork, 0);
+            for (size_t c = 0; c < classes.size(); ++c) {
+                const AcctClass& q = classes[c];
+                cudaStream_t s = c % nstream ? SC.chst[c % nstream - 1] : st;
+                AF.order = AD.order = b->asset_idx ? PK.order + q.first : nullptr;
+                if (fp64) launch_acct_admm(AD, q.shape, q.count, s);
+                else launch_acct_admm(AF, q.shape, q.count, s);
+            }
+            for (int c = 1; c < nstream; ++c) {
+                cudaEventRecord(SC.ev_join[c - 1], SC.chst[c - 1]);
+                cudaStreamWaitEvent(st, SC.ev_join[c - 1], 0);
+            }
+        });
+    };
+    if (acct) {
+        if (b->asset_idx)
+            SC.prof.run(PRISM_K_OTHER, 1, st, [&] {
+                launch_member_lists(M, Npad, S, member, U.d_sec_start, PA.offsets, PK.plist, PK.psec, st);
+            });
+        run_acct(0, o->eps_admm, o->max_iter);
+    } else if (fp64) {
         // PLAIN_FP64: every iteration of the account in one FP64 launch (block_admm.cu)
         P64.resume = 0;
         SC.prof.run(PRISM_K_BLOCK, 1, st, [&] { launch_block_admm(P64, blk_grid(P64), st); });
@@ -1128,7 +1270,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         PK.resume = 0;
         SC.prof.run(PRISM_K_BLOCK, 1, st, [&] { launch_block_admm(PK, blk_grid(PK), st); });
     }
-    if ((fp64 || packed) && D.stats) {
+    if ((fp64 || packed) && !acct && D.stats) {
         // diagnostics: ns per phase summed over accounts, iterations, projection evaluations
         unsigned long long h[8] = {};
         BlkArgs<float> DP = PK;
@@ -1212,7 +1354,9 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         PRISM_CUDA_TRY(cudaMemcpyAsync(P.done, done.data(), M * 4, cudaMemcpyHostToDevice, st));
         PRISM_CUDA_TRY(cudaStreamSynchronize(st));
         int more = 0;
-        if (fp64) {
+        if (acct) {
+            run_acct(1, o->eps_admm * (retry == 0 ? 0.1 : 0.01), o->max_iter * (retry + 2));
+        } else if (fp64) {
             // continue the FP64 iterations of the accounts sent back, to a tighter target
             BlkArgs<double> R = P64;
             R.resume = 1;

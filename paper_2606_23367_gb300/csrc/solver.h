@@ -116,6 +116,7 @@ struct Dev {
     // no loads and its first bounded wait, on a barrier nothing completes, runs out after this
     // many ns; 0 in every normal call
     unsigned long long stall_ns = 0;
+    unsigned long long* t0 = nullptr;   // device clock when the state was initialised (time budgets)
 };
 
 // launchers (admm.cu)
