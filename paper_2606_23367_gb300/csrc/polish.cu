@@ -65,6 +65,11 @@ __device__ __forceinline__ void entry_pieces(const PolDev& P, size_t e, Pieces& 
     }
 }
 
+// The linear term of entry e (position p): mu and the account's tilt of it.
+__device__ __forceinline__ double mu_at(const PolDev& P, size_t e, int p) {
+    return P.tilt ? P.mu64[p] + P.tilt[e] : P.mu64[p];
+}
+
 // The per-entry inputs of the checks, loaded together so that one thread has many
 // independent loads in flight (the int8 state stores would otherwise order them).
 struct EntryRaw {
@@ -75,7 +80,7 @@ struct EntryRaw {
 __device__ __forceinline__ void load_raw(const PolDev& P, size_t base, int p, EntryRaw& r) {
     const size_t e = base + p;
     r.w0 = P.w0[e]; r.lo = P.lo[e]; r.up = P.up[e]; r.c = P.c[e];
-    r.W = P.W[e]; r.d = P.d64[p]; r.mu = P.mu64[p]; r.bn1 = P.Bn1[p];
+    r.W = P.W[e]; r.d = P.d64[p]; r.mu = mu_at(P, e, p); r.bn1 = P.Bn1[p];
     r.code = P.st[e];
     r.sec = P.sector[p];
     r.pw = P.pw_idx ? P.pw_idx[e] : -1;
@@ -580,7 +585,7 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
                 const double tv = fabs(wv - pc.w0);
                 ca += tv;
                 ta += tv;
-                oa += P.d64[p] * wv * wv - P.mu64[p] * wv + phi_value(pc, wv);
+                oa += P.d64[p] * wv * wv - mu_at(P, base + p, p) * wv + phi_value(pc, wv);
                 nn += (wv != 0.0);
             }
         };
@@ -728,7 +733,7 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
             entry_pieces(P, e, pc);
             const int seg = P.st[e] - ST_FREE;
             double* Yq = F.Y + (size_t)q * YS;
-            Yq[0] = P.mu64[p] - pc.sl[seg] - 2.0 * bf;
+            Yq[0] = mu_at(P, e, p) - pc.sl[seg] - 2.0 * bf;
             Yq[COL_W] = 0.0;
             F.dinv[q] = 1.0 / P.d64[p];
             if (q < FS) sh.dinvf_s[q] = float(F.dinv[q]);
@@ -1017,7 +1022,8 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
             t.pw = P.pw_idx ? P.pw_idx[e] : -1;
             t.sec = P.sector[p];
             t.w0 = P.w0f[e]; t.lo = P.lof[e]; t.up = P.upf[e]; t.c = P.cf[e];
-            t.mu = P.mu32[p]; t.bn1 = P.Bn1f[p];
+            t.mu = P.tiltf ? P.mu32[p] + P.tiltf[e] : P.mu32[p];
+            t.bn1 = P.Bn1f[p];
         };
         TileIn cur{}, nxt{};
         if (warp < ntiles) load_tile(warp, cur);
@@ -1232,7 +1238,7 @@ __global__ void __launch_bounds__(PB) k_diag_only(PolDev P) {
         sw += wv;
         rb = fmax(rb, fmax(P.lo[e] - wv, wv - P.up[e]));
         tu += fabs(wv - pc.w0);
-        ol += P.d64[p] * wv * wv - P.mu64[p] * wv + phi_value(pc, wv);
+        ol += P.d64[p] * wv * wv - mu_at(P, e, p) * wv + phi_value(pc, wv);
     }
     sw = warp_sum(sw); rb = warp_max(rb); ol = warp_sum(ol); tu = warp_sum(tu);
     if (lane == 0) { red[warp][0] = sw; red[warp][1] = rb; red[warp][2] = ol; red[warp][3] = tu; }

@@ -18,6 +18,8 @@ struct PolDev {
     const double* Bn1 = nullptr;        // sum_k |B_ik| per asset (error bound of that product)
     const float* Bn1f = nullptr;        // its FP32 copy
     const float* mu32 = nullptr;
+    double* tilt = nullptr;             // M x Npad shift of mu per entry (and its FP32 copy), or null
+    float* tiltf = nullptr;
     const float* w0f = nullptr;         // FP32 copies of the per-entry data (M x Npad)
     const float* lof = nullptr;
     const float* upf = nullptr;

@@ -116,7 +116,9 @@ void release_cache(prism_universe* uh);
 // ---------------------------------------------------------------------------
 // pack / validate
 // ---------------------------------------------------------------------------
-enum : int { ERR_INDEX = 1, ERR_NONFINITE = 2, ERR_BOUNDS = 4, ERR_DUP = 8, ERR_COST = 16, ERR_LEN = 32 };
+enum : int { ERR_INDEX = 1, ERR_NONFINITE = 2, ERR_BOUNDS = 4, ERR_DUP = 8, ERR_COST = 16, ERR_LEN = 32,
+              ERR_LOT_OFFSETS = 64, ERR_LOT_COUNT = 128, ERR_LOT_LOWER = 256, ERR_LOT_DATA = 512, ERR_LOT_SUM = 1024,
+              ERR_BENCH = 2048, ERR_TILT = 4096 };
 
 struct PackArgs {
     int M, N, Npad;
@@ -297,76 +299,184 @@ __global__ void k_capacity(int S, int N, int Npad, const int* sec_start, const d
 }
 
 // ---------------------------------------------------------------------------
-// tax lots: convex piecewise-linear transition cost (lot-LP partial minimum)
+// tax lots (convex piecewise-linear transition cost, the lot-LP's partial minimum) and tilts
+//
+// One thread per entry with lots builds its row of breakpoints and slopes. The rows used to be built on
+// the host, entry by entry, and copied: 25 of the 52 ms of a 200 x 1,924 tax-lot book, and 5 of the
+// 18 ms of a 64 x 2,000 book with a benchmark, whose tilt 2 Sigma w_b needs two passes over the factors.
 // ---------------------------------------------------------------------------
-struct PwlRow {
-    double bp[MAXBP];
-    double sl[MAXBP - 1];
-    int nb;
-    double phi_lo;
+struct CostArgs {
+    int M, N, Npad, K;
+    int64_t nnz, n_lots;
+    const int64_t* offsets;
+    const int32_t* asset_idx;
+    const int* inv_perm;
+    const double *w0, *lo, *up, *tc;    // ragged
+    const int64_t* lot_off;             // nnz + 1, or null
+    const double *lot_size, *lot_kappa;
+    const double *mu_tilt, *w_bench;    // ragged, or null
+    const double *B, *f, *d;            // sorted positions
+    double* h;                          // M x K: F B' w_b
+    double* tilt;                       // M x Npad, and its FP32 copy
+    float* tiltf;
+    int tilt_rows;                      // 1: entries with a tilt carry it in a row (row n_lots + e)
+    int* pw_idx;                        // M x Npad, -1 beforehand; or null
+    double *bp, *sl, *phi_lo;
+    float *bpf, *slf;
+    int* nbp;
+    int* err;                           // [0] flags, [1] rows written
 };
 
-// phi(x) = c (x - w0) + G(max(S*, w0 - x)), G(S) = 2 c S + cheapest-first lot cost of S.
-static double lot_phi(double x, double w0, double c, const std::vector<std::pair<double, double>>& lots) {
+__device__ __forceinline__ int account_of(const int64_t* offsets, int M, int64_t e) {
+    int lo = 0, hi = M;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (offsets[mid] <= e) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+// phi(x) = c (x - w0) + G(max(S*, w0 - x)), G(S) = 2 c S + cheapest-first lot cost of S; lots sorted by kappa
+__device__ double lot_phi(double x, double w0, double c, int L, const double* sz, const double* ka) {
     double sstar = 0.0;
-    for (auto& l : lots) if (2.0 * c + l.second < 0.0) sstar += l.first;
-    double S = std::max(sstar, w0 - x);
+    for (int j = 0; j < L; ++j) if (2.0 * c + ka[j] < 0.0) sstar += sz[j];
+    const double S = fmax(sstar, w0 - x);
     double g = 2.0 * c * S, rem = S;
-    for (size_t j = 0; j < lots.size() && rem > 0; ++j) {
-        double take = (j + 1 < lots.size()) ? std::min(rem, lots[j].first) : rem;
-        g += lots[j].second * take;
+    for (int j = 0; j < L && rem > 0; ++j) {
+        const double take = (j + 1 < L) ? fmin(rem, sz[j]) : rem;
+        g += ka[j] * take;
         rem -= take;
     }
     return c * (x - w0) + g;
 }
 
-static bool build_pwl(double w0, double lo, double up, double c, std::vector<std::pair<double, double>> lots,
-                      PwlRow& row) {
-    std::stable_sort(lots.begin(), lots.end(),
-                     [](const std::pair<double, double>& a, const std::pair<double, double>& b) { return a.second < b.second; });
-    // kinks over the real line with the slope to their right
-    std::vector<double> kinks;
-    std::vector<double> right_slope;
-    const int L = (int)lots.size();
-    int js = 0;
-    while (js < L && 2.0 * c + lots[js].second < 0.0) ++js;
-    std::vector<double> slopes;   // left to right
-    if (js < L) {
+__global__ void k_costs(CostArgs A) {
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= A.nnz) return;
+    const int a = A.asset_idx ? account_of(A.offsets, A.M, e) : int(e / A.N);
+    const int i = A.asset_idx ? A.asset_idx[e] : int(e - (int64_t)a * A.N);
+    if (i < 0 || i >= A.N) return;                          // (flagged by the pack)
+    const size_t at = (size_t)a * A.Npad + A.inv_perm[i];
+    double t = 0.0;
+    if (A.mu_tilt) t = A.mu_tilt[e];
+    if (A.w_bench) {
+        const double wb = A.w_bench[e];
+        if (!isfinite(wb)) { atomicOr(A.err, ERR_BENCH); return; }
+        const double* Bi = A.B + (size_t)A.inv_perm[i] * A.K;
+        double acc = A.d[A.inv_perm[i]] * wb;
+        for (int k = 0; k < A.K; ++k) acc += Bi[k] * A.h[(size_t)a * A.K + k];
+        t += 2.0 * acc;
+    }
+    if (!isfinite(t)) { atomicOr(A.err, ERR_TILT); return; }
+    if (A.tilt) { A.tilt[at] = t; A.tiltf[at] = float(t); }
+    const double shift = A.tilt_rows ? t : 0.0;
+    int64_t l0 = 0, l1 = 0;
+    if (A.lot_off) {
+        l0 = A.lot_off[e]; l1 = A.lot_off[e + 1];
+        if (l0 < 0 || l1 < l0 || l1 > A.n_lots) { atomicOr(A.err, ERR_LOT_OFFSETS); return; }
+    }
+    if (l1 == l0 && shift == 0.0) return;
+    const double w0 = A.w0[e], lo = A.lo[e], up = A.up[e], c = A.tc[e];
+    double bp[MAXBP], sl[MAXBP - 1], phi;
+    int nb;
+    int64_t row;
+    if (l1 > l0) {
+        row = l0;                                           // unique: its lots are its own
+        const int L = int(l1 - l0 > MAXLOT ? MAXLOT + 1 : l1 - l0);
+        if (L > MAXLOT) { atomicOr(A.err, ERR_LOT_COUNT); return; }
+        if (lo < 0) { atomicOr(A.err, ERR_LOT_LOWER); return; }
+        double sz[MAXLOT], ka[MAXLOT], hs = 0;
+        for (int q = 0; q < L; ++q) {
+            const double s = A.lot_size[l0 + q], k = A.lot_kappa[l0 + q];
+            if (!(s >= 0) || !isfinite(k)) { atomicOr(A.err, ERR_LOT_DATA); return; }
+            hs += s;
+            int j = q;                                      // stable insertion by kappa
+            for (; j > 0 && ka[j - 1] > k; --j) { ka[j] = ka[j - 1]; sz[j] = sz[j - 1]; }
+            ka[j] = k; sz[j] = s;
+        }
+        if (fabs(hs - w0) > 1e-9 * fmax(1.0, fabs(w0))) { atomicOr(A.err, ERR_LOT_SUM); return; }
+        // kinks in increasing order; slope j is that left of kink j, c right of the last
+        int js = 0;
+        while (js < L && 2.0 * c + ka[js] < 0.0) ++js;
+        const int nk = L - js;
+        double kink[MAXLOT];
         double H = 0.0;
-        for (int j = 0; j < js; ++j) H += lots[j].first;
-        // slope right of w0 - S* is c; left of it the lots js, js+1, ... are sold in turn
-        double x = w0 - H;
-        kinks.push_back(x);
-        double Hj = H;
-        std::vector<double> xs{x};
-        for (int j = js; j < L - 1; ++j) { Hj += lots[j].first; xs.push_back(w0 - Hj); }
-        // xs decreasing; slopes left of xs[q] = -c - kappa[js + q]
-        kinks.assign(xs.rbegin(), xs.rend());
-        for (int j = L - 1; j >= js; --j) slopes.push_back(-c - lots[j].second);
-        slopes.push_back(c);
+        for (int j = 0; j < js; ++j) H += sz[j];
+        for (int j = 0; j < nk; ++j) {
+            kink[nk - 1 - j] = w0 - H;
+            H += sz[js + j];
+        }
+        auto slope = [&](int q) { return q < nk ? -c - ka[L - 1 - q] : c; };
+        phi = lot_phi(lo, w0, c, L, sz, ka);
+        nb = 1;
+        bp[0] = lo;
+        if (up > lo) {
+            // the kinks and w0 inside the box, sorted, each once
+            bool held = w0 > lo && w0 < up;
+            for (int j = 0; j <= nk; ++j) {
+                if (held && (j == nk || w0 <= kink[j])) {
+                    if (w0 > bp[nb - 1]) bp[nb++] = w0;
+                    held = false;
+                }
+                if (j < nk && kink[j] > lo && kink[j] < up && kink[j] > bp[nb - 1]) bp[nb++] = kink[j];
+            }
+            bp[nb++] = up;
+            for (int j = 0; j + 1 < nb; ++j) {
+                const double mid = 0.5 * (bp[j] + bp[j + 1]);
+                int q = 0;
+                while (q < nk && kink[q] <= mid) ++q;
+                sl[j] = slope(q);
+            }
+        }
     } else {
-        slopes.push_back(c);
+        // the plain L1 cost as a row: breakpoints l, w0 (inside the box), u
+        row = A.n_lots + e;
+        phi = c * fabs(lo - w0);
+        if (!(up > lo)) {
+            nb = 1; bp[0] = lo;
+        } else if (w0 > lo && w0 < up) {
+            nb = 3; bp[0] = lo; bp[1] = w0; bp[2] = up; sl[0] = -c; sl[1] = c;
+        } else {
+            nb = 2; bp[0] = lo; bp[1] = up; sl[0] = (w0 <= lo) ? c : -c;
+        }
     }
-    if (!(up > lo)) {
-        row.nb = 1; row.bp[0] = lo; row.phi_lo = lot_phi(lo, w0, c, lots);
-        return true;
+    // a term -t w shifts every slope by -t
+    for (int j = 0; j + 1 < nb; ++j) {
+        const double s = sl[j] - shift;
+        A.sl[row * (MAXBP - 1) + j] = s;
+        A.slf[row * (MAXBP - 1) + j] = float(s);
     }
-    std::vector<double> pts{lo};
-    for (double x : kinks) if (x > lo && x < up) pts.push_back(x);
-    if (w0 > lo && w0 < up) pts.push_back(w0);
-    std::sort(pts.begin(), pts.end());
-    pts.erase(std::unique(pts.begin(), pts.end()), pts.end());
-    pts.push_back(up);
-    if ((int)pts.size() > MAXBP) return false;
-    row.nb = (int)pts.size();
-    for (int j = 0; j < row.nb; ++j) row.bp[j] = pts[j];
-    for (int j = 0; j + 1 < row.nb; ++j) {
-        double mid = 0.5 * (pts[j] + pts[j + 1]);
-        int q = int(std::upper_bound(kinks.begin(), kinks.end(), mid) - kinks.begin());
-        row.sl[j] = slopes[q];
+    for (int j = 0; j < nb; ++j) {
+        A.bp[row * MAXBP + j] = bp[j];
+        A.bpf[row * MAXBP + j] = float(bp[j]);
     }
-    row.phi_lo = lot_phi(lo, w0, c, lots);
-    return true;
+    A.phi_lo[row] = phi - shift * bp[0];
+    A.nbp[row] = nb;
+    A.pw_idx[at] = (int)row;
+    if (A.err[1] == 0) A.err[1] = 1;
+}
+
+// F B' w_b of each account, FP64: a block per account, its warps over the entries, a lane per factor
+__global__ void __launch_bounds__(256) k_bench_factors(CostArgs A) {
+    const int a = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5;
+    __shared__ double part[8][KMAX];
+    double a0 = 0.0, a1 = 0.0;
+    for (int64_t e = A.offsets[a] + warp; e < A.offsets[a + 1]; e += NW) {
+        const int i = A.asset_idx ? A.asset_idx[e] : int(e - A.offsets[a]);
+        if (i < 0 || i >= A.N) continue;
+        const double wb = A.w_bench[e];
+        const double* Bi = A.B + (size_t)A.inv_perm[i] * A.K;
+        if (lane < A.K) a0 += Bi[lane] * wb;
+        if (lane + 32 < A.K) a1 += Bi[lane + 32] * wb;
+    }
+    part[warp][lane] = a0;
+    part[warp][lane + 32] = a1;
+    __syncthreads();
+    for (int k = threadIdx.x; k < A.K; k += blockDim.x) {
+        double s = 0.0;
+        for (int w = 0; w < NW; ++w) s += part[w][k];
+        A.h[(size_t)a * A.K + k] = A.f[k] * s;
+    }
 }
 
 template <typename T>
@@ -416,7 +526,7 @@ static double batched_iteration_us(int M, int N, bool bf16, bool staged) {
 }
 
 static bool acct_route(const prism_solve_opts& o, bool plain, bool fp64, bool bf16, bool ragged, int M, int N, int K,
-                       bool pw, bool fac, bool cap, const std::vector<int64_t>& offs, std::vector<AcctClass>& classes,
+                       bool pw, bool tilt, bool fac, bool cap, const std::vector<int64_t>& offs, std::vector<AcctClass>& classes,
                        std::vector<int>& order) {
     // an option that names a form of the batched kernels keeps the book on them, and so does the
     // failure-path test of their tensor-core waits
@@ -452,7 +562,7 @@ static bool acct_route(const prism_solve_opts& o, bool plain, bool fp64, bool bf
     }
     // single accounts and the packed layout have no batched form
     if (plain || o.ragged_layout == 2) return true;
-    return us <= batched_iteration_us(M, N, bf16, pw || cap || fac);
+    return us <= batched_iteration_us(M, N, bf16, pw || tilt || cap || fac);
 }
 
 // ---------------------------------------------------------------------------
@@ -480,115 +590,11 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         if (offs[a + 1] - offs[a] > N) { set_error("account longer than the universe"); return PRISM_ERR_ARGUMENT; }
     }
     const int64_t nnz = offs[M];
-    // ---- lots (host-side construction of the piecewise-linear tables)
-    std::vector<PwlRow> pwl;
-    std::vector<int> pw_of_entry;   // ragged entry -> pw row or -1
-    const bool has_lots = b->lot_offsets != nullptr;
-    if (has_lots) {
-        std::vector<int64_t> lo_off;
-        std::vector<double> lsz, lka, w0h, loh, uph, tch;
-        if ((rc = to_host(b->lot_offsets, (size_t)nnz + 1, lo_off))) return rc;
-        const int64_t nl = lo_off[nnz];
-        if ((rc = to_host(b->lot_size, (size_t)nl, lsz)) || (rc = to_host(b->lot_kappa, (size_t)nl, lka)) ||
-            (rc = to_host(b->w0, (size_t)nnz, w0h)) || (rc = to_host(b->lower, (size_t)nnz, loh)) ||
-            (rc = to_host(b->upper, (size_t)nnz, uph)) || (rc = to_host(b->tc, (size_t)nnz, tch)))
-            return rc;
-        pw_of_entry.assign(nnz, -1);
-        for (int64_t e = 0; e < nnz; ++e) {
-            const int64_t l0 = lo_off[e], l1 = lo_off[e + 1];
-            if (l1 < l0) { set_error("lot_offsets must be nondecreasing"); return PRISM_ERR_ARGUMENT; }
-            if (l1 == l0) continue;
-            if (l1 - l0 > MAXLOT) { set_error("more than 4 lots on one entry"); return PRISM_ERR_UNSUPPORTED; }
-            if (loh[e] < 0) { set_error("lots need lower >= 0"); return PRISM_ERR_ARGUMENT; }
-            std::vector<std::pair<double, double>> lots;
-            double hs = 0;
-            for (int64_t q = l0; q < l1; ++q) {
-                if (!(lsz[q] >= 0) || !std::isfinite(lka[q])) { set_error("bad lot data"); return PRISM_ERR_ARGUMENT; }
-                lots.push_back({lsz[q], lka[q]});
-                hs += lsz[q];
-            }
-            if (std::fabs(hs - w0h[e]) > 1e-9 * std::max(1.0, std::fabs(w0h[e]))) {
-                set_error("lot sizes of an entry must sum to its w0");
-                return PRISM_ERR_ARGUMENT;
-            }
-            PwlRow row;
-            if (!build_pwl(w0h[e], loh[e], uph[e], tch[e], lots, row)) {
-                set_error("too many breakpoints in a lot cost");
-                return PRISM_ERR_UNSUPPORTED;
-            }
-            pw_of_entry[e] = (int)pwl.size();
-            pwl.push_back(row);
-        }
-    }
-    // Tilts of the linear term (Eq. 1's per-account return tilt, and the benchmark's 2 Sigma w_b):
-    // a term -t_i w_i is linear, so it shifts every slope of phi_i by -t_i; entries with a tilt
-    // carry it in a piecewise-linear cost row (their lot row when they have lots)
-    const bool has_tilt = b->mu_tilt || b->w_bench;
-    if (has_tilt) {
-        std::vector<double> tilt((size_t)nnz, 0.0), w0h, loh, uph, tch, tmp;
-        std::vector<int32_t> aidx;
-        if ((rc = to_host(b->w0, (size_t)nnz, w0h)) || (rc = to_host(b->lower, (size_t)nnz, loh)) ||
-            (rc = to_host(b->upper, (size_t)nnz, uph)) || (rc = to_host(b->tc, (size_t)nnz, tch)))
-            return rc;
-        if (b->asset_idx && (rc = to_host(b->asset_idx, (size_t)nnz, aidx))) return rc;
-        auto asset = [&](int a, int64_t e) { return b->asset_idx ? int(aidx[e]) : int(e - offs[a]); };
-        if (b->mu_tilt) {
-            if ((rc = to_host(b->mu_tilt, (size_t)nnz, tmp))) return rc;
-            for (int64_t e = 0; e < nnz; ++e) tilt[e] = tmp[e];
-        }
-        if (b->w_bench) {
-            // 2 Sigma_a w_b over the account's own names: 2 (B (F (B' w_b)) + D w_b), FP64
-            std::vector<double> wb, Bh((size_t)U.Npad * K), fh, dh;
-            if ((rc = to_host(b->w_bench, (size_t)nnz, wb)) || (rc = to_host(U.d_B64, (size_t)U.Npad * K, Bh)) ||
-                (rc = to_host(U.d_f64, (size_t)K, fh)) || (rc = to_host(U.d_d64, (size_t)U.Npad, dh)))
-                return rc;
-            std::vector<double> h(K);
-            for (int a = 0; a < M; ++a) {
-                std::fill(h.begin(), h.end(), 0.0);
-                for (int64_t e = offs[a]; e < offs[a + 1]; ++e) {
-                    if (!std::isfinite(wb[e])) { set_error("w_bench must be finite"); return PRISM_ERR_ARGUMENT; }
-                    const int i = asset(a, e);
-                    if (i < 0 || i >= N) { set_error("asset index out of range"); return PRISM_ERR_ARGUMENT; }
-                    const double* Bi = &Bh[(size_t)U.inv_perm[i] * K];
-                    for (int k = 0; k < K; ++k) h[k] += Bi[k] * wb[e];
-                }
-                for (int k = 0; k < K; ++k) h[k] *= fh[k];
-                for (int64_t e = offs[a]; e < offs[a + 1]; ++e) {
-                    const int p = U.inv_perm[asset(a, e)];
-                    const double* Bi = &Bh[(size_t)p * K];
-                    double acc = dh[p] * wb[e];
-                    for (int k = 0; k < K; ++k) acc += Bi[k] * h[k];
-                    tilt[e] += 2.0 * acc;
-                }
-            }
-        }
-        if (pw_of_entry.empty()) pw_of_entry.assign(nnz, -1);
-        for (int64_t e = 0; e < nnz; ++e) {
-            const double t = tilt[e];
-            if (!std::isfinite(t)) { set_error("mu_tilt must be finite"); return PRISM_ERR_ARGUMENT; }
-            if (t == 0.0) continue;
-            if (pw_of_entry[e] < 0) {
-                // the plain L1 cost as a row: breakpoints l, w0 (inside the box), u
-                PwlRow row;
-                const double lo = loh[e], up = uph[e], w0 = w0h[e], c = tch[e];
-                row.phi_lo = c * std::fabs(lo - w0);
-                if (!(up > lo)) {
-                    row.nb = 1; row.bp[0] = lo;
-                } else if (w0 > lo && w0 < up) {
-                    row.nb = 3; row.bp[0] = lo; row.bp[1] = w0; row.bp[2] = up; row.sl[0] = -c; row.sl[1] = c;
-                } else {
-                    row.nb = 2; row.bp[0] = lo; row.bp[1] = up; row.sl[0] = (w0 <= lo) ? c : -c;
-                }
-                pw_of_entry[e] = (int)pwl.size();
-                pwl.push_back(row);
-            }
-            PwlRow& row = pwl[pw_of_entry[e]];
-            for (int j = 0; j + 1 < row.nb; ++j) row.sl[j] -= t;
-            row.phi_lo -= t * row.bp[0];
-        }
-    }
-    const int n_pw = (int)pwl.size();
-    const bool has_pw = has_lots || n_pw > 0;
+    // ---- lots and tilts (see k_costs)
+    const bool has_lots = b->lot_offsets != nullptr, has_tilt = b->mu_tilt || b->w_bench;
+    int64_t n_lots = 0;
+    if (has_lots) PRISM_CUDA_TRY(cudaMemcpy(&n_lots, b->lot_offsets + nnz, sizeof(int64_t), cudaMemcpyDefault));
+    if (n_lots < 0) { set_error("lot_offsets must be nondecreasing"); return PRISM_ERR_ARGUMENT; }
     // factor-exposure bounds: validated on the host, any finite one turns the block on
     std::vector<double> flo_h, fhi_h;
     bool has_fac_in = false;
@@ -613,8 +619,14 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     // ---- which iterations: account-resident (acct_admm.cuh) where its accounts fit and it is the faster
     std::vector<AcctClass> classes;
     std::vector<int> order_h;
-    const bool acct = acct_route(*o, plain, fp64, batched_mode_bf16, b->asset_idx != nullptr, M, N, K, has_pw, has_fac_in,
-                                 b->turnover_cap != nullptr, offs, classes, order_h);
+    const bool acct = acct_route(*o, plain, fp64, batched_mode_bf16, b->asset_idx != nullptr, M, N, K, has_lots, has_tilt,
+                                 has_fac_in, b->turnover_cap != nullptr, offs, classes, order_h);
+    // the account-resident kernel takes a tilt as a shift of mu, the batched ones as cost rows
+    const bool tilt_rows = has_tilt && !acct;
+    const bool has_pw = has_lots || tilt_rows;
+    const int64_t n_pw64 = n_lots + (tilt_rows ? nnz : 0);
+    if (n_pw64 > INT32_MAX) { set_error("too many tax lots"); return PRISM_ERR_UNSUPPORTED; }
+    const int n_pw = (int)n_pw64;
     if (acct) packed = false;
     const bool lists = packed || (acct && b->asset_idx);   // per-account position lists are needed
     // ---- workspace layout
@@ -690,6 +702,12 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         BD.pw_slf = A.take<float>((size_t)std::max(n_pw, 1) * (MAXBP - 1));
         BD.pw_nbp = A.take<int>((size_t)std::max(n_pw, 1));
         stage[6] = A.take<double>((size_t)std::max(n_pw, 1));   // phi_lo
+        stage[7] = A.take<int64_t>(has_lots ? (size_t)nnz + 1 : 0);
+        stage[8] = A.take<double>((size_t)n_lots); stage[9] = A.take<double>((size_t)n_lots);
+        stage[10] = A.take<double>(b->mu_tilt ? (size_t)nnz : 0); stage[11] = A.take<double>(b->w_bench ? (size_t)nnz : 0);
+        stage[12] = A.take<double>(b->w_bench ? (size_t)M * K : 0);
+        const size_t nt64 = (has_tilt && !tilt_rows) ? MN : 0;
+        P.tilt = A.take<double>(nt64); P.tiltf = A.take<float>(nt64);
         // FP64 iteration state of PLAIN_FP64 (z, y, X/v per entry; penalty and cap multiplier)
         const size_t n64 = fp64 ? MN : 0;
         P64.z = A.take<double>(n64); P64.y = A.take<double>(n64); P64.X = A.take<double>(n64);
@@ -714,7 +732,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     std::memset((void*)&D, 0, sizeof(Dev));   // padding bytes take part in the graph-reuse test
     PolDev P;
     BatchDev BD;
-    void* stage[7];
+    void* stage[13];
     int *member, *err, *pwidx;
     double* ragged_out;
     {
@@ -843,42 +861,50 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         }
         PRISM_CUDA_TRY(cudaStreamSynchronize(st));
     }
-    // lot tables
-    std::vector<double> h_phi;
-    if (has_pw) {
-        std::vector<double> bp((size_t)std::max(n_pw, 1) * MAXBP, 0.0), sl((size_t)std::max(n_pw, 1) * (MAXBP - 1), 0.0);
-        std::vector<float> bpf(bp.size()), slf(sl.size());
-        std::vector<int> nb(std::max(n_pw, 1), 1);
-        h_phi.assign(std::max(n_pw, 1), 0.0);
-        for (int r = 0; r < n_pw; ++r) {
-            nb[r] = pwl[r].nb;
-            h_phi[r] = pwl[r].phi_lo;
-            for (int j = 0; j < pwl[r].nb; ++j) { bp[(size_t)r * MAXBP + j] = pwl[r].bp[j]; bpf[(size_t)r * MAXBP + j] = float(pwl[r].bp[j]); }
-            for (int j = 0; j + 1 < pwl[r].nb; ++j) { sl[(size_t)r * (MAXBP - 1) + j] = pwl[r].sl[j]; slf[(size_t)r * (MAXBP - 1) + j] = float(pwl[r].sl[j]); }
+    // lots and tilts
+    if (has_lots || has_tilt) {
+        CostArgs CA = {};
+        CA.M = M; CA.N = N; CA.Npad = Npad; CA.K = K; CA.nnz = nnz; CA.n_lots = n_lots;
+        CA.offsets = PA.offsets; CA.asset_idx = PA.asset_idx; CA.inv_perm = U.d_inv_perm;
+        CA.w0 = PA.w0; CA.lo = PA.lo; CA.up = PA.up; CA.tc = PA.tc;
+        if (has_lots) {
+            CA.lot_off = (const int64_t*)stage_in(b->lot_offsets, stage[7], (nnz + 1) * sizeof(int64_t));
+            CA.lot_size = (const double*)stage_in(b->lot_size, stage[8], n_lots * 8);
+            CA.lot_kappa = (const double*)stage_in(b->lot_kappa, stage[9], n_lots * 8);
         }
-        // per sorted entry index of the table row
-        std::vector<int> pwidx_h(MN, -1);
-        std::vector<int32_t> aidx;
-        if (b->asset_idx && (rc = to_host(b->asset_idx, (size_t)nnz, aidx))) return rc;
-        for (int a = 0; a < M; ++a)
-            for (int64_t e = offs[a]; e < offs[a + 1]; ++e) {
-                int i = b->asset_idx ? aidx[e] : int(e - offs[a]);
-                if (i < 0 || i >= N) { set_error("asset index out of range"); return PRISM_ERR_ARGUMENT; }
-                pwidx_h[(size_t)a * Npad + U.inv_perm[i]] = pw_of_entry[e];
-            }
-        PRISM_CUDA_TRY(cudaMemcpyAsync(pwidx, pwidx_h.data(), MN * 4, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaMemcpyAsync(BD.pw_bp, bp.data(), bp.size() * 8, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaMemcpyAsync(BD.pw_sl, sl.data(), sl.size() * 8, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaMemcpyAsync(BD.pw_bpf, bpf.data(), bpf.size() * 4, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaMemcpyAsync(BD.pw_slf, slf.data(), slf.size() * 4, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaMemcpyAsync(BD.pw_nbp, nb.data(), nb.size() * 4, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaMemcpyAsync(stage[6], h_phi.data(), h_phi.size() * 8, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaStreamSynchronize(st));
+        if (b->mu_tilt) CA.mu_tilt = (const double*)stage_in(b->mu_tilt, stage[10], nnz * 8);
+        if (b->w_bench) CA.w_bench = (const double*)stage_in(b->w_bench, stage[11], nnz * 8);
+        CA.B = U.d_B64; CA.f = U.d_f64; CA.d = U.d_d64; CA.h = (double*)stage[12];
+        CA.tilt_rows = tilt_rows;
+        if (has_tilt && !tilt_rows) {
+            CA.tilt = P.tilt; CA.tiltf = P.tiltf;
+            cudaMemsetAsync(P.tilt, 0, MN * 8, st);
+            cudaMemsetAsync(P.tiltf, 0, MN * 4, st);
+        }
+        CA.pw_idx = pwidx; CA.bp = BD.pw_bp; CA.sl = BD.pw_sl; CA.phi_lo = (double*)stage[6];
+        CA.bpf = BD.pw_bpf; CA.slf = BD.pw_slf; CA.nbp = BD.pw_nbp; CA.err = err;
+        if (pwidx) cudaMemsetAsync(pwidx, 0xff, MN * 4, st);
+        SC.prof.run(PRISM_K_PACK, b->w_bench ? 2 : 1, st, [&] {
+            if (b->w_bench) k_bench_factors<<<M, 256, 0, st>>>(CA);
+            if (nnz > 0) k_costs<<<(unsigned)cdiv64(nnz, 128), 128, 0, st>>>(CA);
+        });
     }
     {
-        int herr = 0;
-        PRISM_CUDA_TRY(cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, st));
+        int flags[2] = {0, 0};
+        PRISM_CUDA_TRY(cudaMemcpyAsync(flags, err, 8, cudaMemcpyDeviceToHost, st));
         PRISM_CUDA_TRY(cudaStreamSynchronize(st));
+        const int herr = flags[0];
+        if (!has_lots && !flags[1]) pwidx = nullptr;      // every tilt is zero: plain costs throughout
+        struct { int bit, code; const char* text; } lot_errors[] = {
+            {ERR_LOT_OFFSETS, PRISM_ERR_ARGUMENT, "lot_offsets must be nondecreasing"},
+            {ERR_LOT_COUNT, PRISM_ERR_UNSUPPORTED, "more than 4 lots on one entry"},
+            {ERR_LOT_LOWER, PRISM_ERR_ARGUMENT, "lots need lower >= 0"},
+            {ERR_LOT_DATA, PRISM_ERR_ARGUMENT, "bad lot data"},
+            {ERR_LOT_SUM, PRISM_ERR_ARGUMENT, "lot sizes of an entry must sum to its w0"},
+            {ERR_BENCH, PRISM_ERR_ARGUMENT, "w_bench must be finite"},
+            {ERR_TILT, PRISM_ERR_ARGUMENT, "mu_tilt must be finite"}};
+        for (auto& q : lot_errors)
+            if (herr & q.bit) { set_error(q.text); return q.code; }
         if (herr) {
             std::string m = "invalid batch input:";
             if (herr & ERR_INDEX) m += " asset index out of range;";
@@ -936,6 +962,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     P.B32 = U.d_B32; P.B32p = U.d_B32p; P.Bn1 = U.d_Bn1; P.Bn1f = U.d_Bn1f; P.mu32 = U.d_mu32;
     P.w0f = BD.w0f; P.lof = BD.lof; P.upf = BD.upf; P.cf = BD.cf;
     P.w0 = BD.w0; P.lo = BD.lo; P.up = BD.up; P.c = BD.c;
+    if (!has_tilt || tilt_rows) { P.tilt = nullptr; P.tiltf = nullptr; }
     P.pw_idx = pwidx; P.pw_bp = BD.pw_bp; P.pw_sl = BD.pw_sl; P.pw_phi_lo = (const double*)stage[6]; P.pw_nbp = BD.pw_nbp;
     P.band_lo = BD.band_lo; P.band_hi = BD.band_hi; P.tau = BD.tau;
     if (BD.has_fac) { P.flo = BD.flo; P.fhi = BD.fhi; P.sflag = D.sflag; }
@@ -1215,6 +1242,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         AF.pw_bp = BD.pw_bpf; AF.pw_sl = BD.pw_slf;
         AF.band_lo = BD.band_lof; AF.band_hi = BD.band_hif;
         AF.z = D.z; AF.y = D.y;
+        AF.tilt = P.tiltf; AD.tilt = P.tilt;
         if (BD.has_cap) AF.tau = BD.tauf;
         if (BD.has_fac) { AF.flo = BD.flof; AF.fhi = BD.fhif; AF.s = D.s; AF.ys = D.ys; }
         AD.B64 = U.d_B64; AD.f = U.d_f64; AD.d = U.d_d64; AD.mu = U.d_mu64;
