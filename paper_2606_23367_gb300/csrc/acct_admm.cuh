@@ -778,6 +778,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
     bool go = true, fresh = true;                     // fresh: a new penalty
     int status = 0;
     bool stopped = false;                             // out of time, still iterating
+    bool watch = false;                               // near the target: the entries' places are followed
+    unsigned held = 0;                                // this thread's entries' places, two bits each
+    int quiet = 0, met = 0;                           // iterations without a change; where the target was met
     int pbuf = 0;
     while (go) {
         if (fresh) {
@@ -942,6 +945,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
         const bool adapt = (it + 1) % A.adapt_every == 0;
         T rp = rps, rd = rds, nx = T(0), nz = T(0), ny = T(0);
         int flags = 0;
+        unsigned codes = 0;
         if (clamped || stale) prox(clamped, nu, th);  // (else zz holds it: nu is where the last evaluation was)
 #pragma unroll
         for (int e = 0; e < E; ++e) {
@@ -956,6 +960,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
                     ny = fmax(ny, fabs(yn));
                 }
                 flags |= !(isfinite(zn) && isfinite(yn));
+                // its place: inside a linear piece above or below w0, or at a breakpoint, and the same one
+                const unsigned code = lin[e] ? (zn > w0[e] ? 1u : 2u) : 0u;
+                codes |= code << (2 * e);
+                if (watch && (((held >> (2 * e)) & 3u) != code || (code == 0 && zn != z[e]))) flags |= 4;
                 z[e] = zn;
                 y[e] = yn;
             }
@@ -997,10 +1005,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
         }
         ++it;
         close = rp;
+        // The residuals having met their target, the account goes on until its entries have kept their places
+        // for A.settle iterations: the polish starts from those places
+        held = codes;
+        quiet = (watch && !(flags & 4)) ? quiet + 1 : 0;
+        watch = A.settle && rp <= T(8) * A.eps && rd <= T(8) * A.eps;
+        if (!met && it >= A.min_iter && rp <= A.eps && rd <= A.eps) met = it;
         // ---- control, the same in every thread
         int newj = j;
         if (flags & 1) { status = PRISM_NUMERICAL_FAILURE; go = false; }
-        else if (it >= A.min_iter && rp <= A.eps && rd <= A.eps) go = false;
+        else if (met && (quiet >= A.settle || it - met >= A.settle_max)) go = false;
         else if (it >= A.max_iter) { status = PRISM_TIMEOUT; go = false; }
         else if (flags & 2) { stopped = true; go = false; }
         else if (adapt) {

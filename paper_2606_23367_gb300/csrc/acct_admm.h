@@ -50,6 +50,8 @@ struct AcctArgs {
     unsigned long long budget_ns = 0;      // time budget from t0 (0: none)
     T alpha = T(1.5), eps = T(5e-4);
     int max_iter = 4000, min_iter = 20, adapt_every = 25;
+    int settle = 0, settle_max = 60;       // iterations without a change of place to wait for once the target
+                                           // is met, and for how many iterations to wait
     int resume = 0;                        // 1: z, y, s, ys and the multipliers continue from the state
     int pw_rows = 0;                       // rows of the cost tables that a CTA can keep in shared memory
 };

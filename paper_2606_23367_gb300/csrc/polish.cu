@@ -28,7 +28,8 @@
 
 namespace prism {
 
-constexpr int PB = 256;             // threads per polish block
+constexpr int PB = 256;             // threads per block of the classification and the diagnostics
+constexpr int PWARPS = 16;          // warps of the largest polish block
 constexpr int ST_FREE = 32;         // state code: free in segment (code - ST_FREE)
 
 // Breakpoints / slopes of phi_i restricted to [l_i, u_i] for one entry (FP64).
@@ -186,12 +187,14 @@ struct PolishShared {
     float Bc[FS][KMAX + 1];               // FP32 rows of B of the first FS free entries
     double Bd[FS][KMAX + 1];              // FP64 rows of B of the first FS free entries
     double Ys[FS][YS];                    // Y rows of the first FS free entries
-    double dinv_s[FS], sig_s[FS];
+    double dinv_s[FS], sig_s[FS], d_s[FS];
     double gF[FS];                        // B_p . (f .* h) of the free entries, for their checks
     float dinvf_s[FS];
     int Fl_s[FS];
     float Ldinv[KMAX];                    // reciprocal of the Cholesky diagonal
     float f32s[KMAX];                     // FP32 factor variances
+    double f64s[KMAX];
+    double ipiv[PMAXROWS], xrow[PMAXROWS];   // 1 / the pivots of the Schur matrix; its solutions
     float T[KMAX][PMAXROWS + 1];          // FP32 Woodbury workspace
     double Sf[PMAXROWS][PMAXROWS + 1];    // Schur matrix after pivoted elimination
     double hA[KMAX], fhA[KMAX], fh[KMAX], t64[KMAX];
@@ -200,11 +203,12 @@ struct PolishShared {
     int order[PMAXROWS], used[PMAXROWS];
     int rows[PMAXROWS];
     int nrows, nF, nNZ, fail, nc, go;
+    unsigned long long hash, past[8];     // of the working set: now, and after the last rounds
     double fhmax_s, quad_s;               // max_k |f_k h_k| and h' F h of the solved point
-    int cntF[PB / 32], cntN[PB / 32];
-    int qp[PB / 32][64];                  // per-warp queue of entries that need FP64 work
-    float qg[PB / 32][64];
-    double sumA[PB / 32], capA[PB / 32], turnA[PB / 32], objA[PB / 32];
+    int cntF[PWARPS], cntN[PWARPS];
+    int qp[PWARPS][64];                  // per-warp queue of entries that need FP64 work
+    float qg[PWARPS][64];
+    double sumA[PWARPS], capA[PWARPS], turnA[PWARPS], objA[PWARPS];
     double lam_s[SMAX];
     double kap_s[KMAX];                   // multipliers of the factor rows (0 off the working set)
     float lam_s32[SMAX];
@@ -214,10 +218,10 @@ struct PolishShared {
     double flo_s[KMAX], fhi_s[KMAX];      // the account's factor-exposure bounds
     double fixS[SMAX];                    // per sector: sum of the fixed weights
     int secF[FS];                         // sector of each of the first FS free entries                  // its FP32 copy (the filter of the checks)
-    double red[PB / 32][8];
+    double red[PWARPS][8];
     double secsum[SMAX];
-    double mmin[PB / 32];
-    int mwho[PB / 32];
+    double mmin[PWARPS];
+    int mwho[PWARPS];
 };
 
 // the free-set data of one account: shared memory when |F| <= FS, else global scratch
@@ -263,6 +267,19 @@ struct WarpQueue {
     }
 };
 
+// A change of item i's state in the working set (entries, then bands, cap and factor rows): added to a hash
+// that tells a set met before. The terms add up in any order.
+__device__ __forceinline__ void note_change(PolishShared& sh, int i, int was, int is) {
+    auto mix = [](unsigned long long x) {                 // (the finaliser of SplitMix64, Steele et al. 2014)
+        x += 0x9e3779b97f4a7c15ull;
+        x = (x ^ (x >> 30)) * 0xbf58476d1ce4e5b9ull;
+        x = (x ^ (x >> 27)) * 0x94d049bb133111ebull;
+        return x ^ (x >> 31);
+    };
+    const unsigned long long b = (unsigned long long)i << 8;
+    atomicAdd(&sh.hash, mix(b | (unsigned char)is) - mix(b | (unsigned char)was));
+}
+
 __device__ __forceinline__ double brow64(const PolDev& P, const PolishShared& sh, const FreeSet& F, int q, int k);
 
 // coefficient of free entry q in working row ``row``: the budget (row -1), the band of sector
@@ -294,13 +311,13 @@ __device__ __forceinline__ double brow64(const PolDev& P, const PolishShared& sh
 // FP64 products with the free rows of B, spread over the whole block (the FP64 pipe
 // runs a warp instruction at the same cost however few of its lanes are active, so the
 // work goes to full warps): fin(q, sum_k B_F[q][k] x[k]) for each free row q, eight lanes per
-// row, and fin(k, sum_q y(q) B_F[q][k]) for each factor k, four lanes per factor. The partial
+// row, and fin(k, sum_q y(q) B_F[q][k]) for each factor k, four or eight lanes per factor. The partial
 // sums are combined in a fixed order. Block-collective (no barrier inside).
-template <class Fin>
+template <int NT, class Fin>
 __device__ __forceinline__ void rows_dot64(const PolDev& P, const PolishShared& sh, const FreeSet& F, int nF,
                                            const double* x, Fin&& fin) {
     const int tid = threadIdx.x, g = tid >> 3, sub = tid & 7, K = P.K;
-    for (int q0 = 0; q0 < nF; q0 += PB / 8) {
+    for (int q0 = 0; q0 < nF; q0 += NT / 8) {
         const int q = q0 + g;
         double acc = 0.0;
         if (q < nF)
@@ -312,14 +329,15 @@ __device__ __forceinline__ void rows_dot64(const PolDev& P, const PolishShared& 
     }
 }
 
-static_assert(PB / 4 >= KMAX, "four lanes per factor");
-template <class Yf, class Fin>
+template <int NT, class Yf, class Fin>
 __device__ __forceinline__ void cols_dot64(const PolDev& P, const PolishShared& sh, const FreeSet& F, int nF,
                                            Yf&& y, Fin&& fin) {
-    const int tid = threadIdx.x, k = tid >> 2, sub = tid & 3, K = P.K;
+    constexpr int L = NT / KMAX;                          // lanes per factor: four or eight
+    const int tid = threadIdx.x, k = tid / L, sub = tid % L, K = P.K;
     double acc = 0.0;
     if (k < K)
-        for (int q = sub; q < nF; q += 4) acc += y(q) * brow64(P, sh, F, q, k);
+        for (int q = sub; q < nF; q += L) acc += y(q) * brow64(P, sh, F, q, k);
+    if (L == 8) acc += __shfl_xor_sync(0xffffffffu, acc, 4);
     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     if (sub == 0 && k < K) fin(k, acc);
@@ -327,10 +345,11 @@ __device__ __forceinline__ void cols_dot64(const PolDev& P, const PolishShared& 
 
 // FP32 Woodbury solve of Sigma_FF x = r for the columns c0..c1 of Y (in: D^{-1} r;
 // out: x). Block-collective.
+template <int NT>
 __device__ __noinline__ void woodbury32(const PolDev& P, PolishShared& sh, const FreeSet& F, int nF, int c0, int c1) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int K = P.K, nc = c1 - c0;
-    for (int e2 = tid; e2 < K * nc; e2 += PB) {
+    for (int e2 = tid; e2 < K * nc; e2 += NT) {
         const int k = e2 / nc, c = c0 + e2 % nc;
         float acc = 0.f;
         for (int q = 0; q < nF; ++q) acc = fmaf(brow32(P, sh, F, q, k), float(F.Y[(size_t)q * YS + c]), acc);
@@ -338,7 +357,7 @@ __device__ __noinline__ void woodbury32(const PolDev& P, PolishShared& sh, const
     }
     __syncthreads();
     // L L' t = T column by column, one warp per column, rows lane and lane + 32 in registers
-    for (int c = warp; c < nc; c += PB / 32) {
+    for (int c = warp; c < nc; c += NT / 32) {
         float v0 = lane < K ? sh.T[lane][c] : 0.f, v1 = lane + 32 < K ? sh.T[lane + 32][c] : 0.f;
         for (int r = 0; r < K; ++r) {
             const float x = __shfl_sync(0xffffffffu, r < 32 ? v0 : v1, r & 31) * sh.Ldinv[r];
@@ -356,7 +375,7 @@ __device__ __noinline__ void woodbury32(const PolDev& P, PolishShared& sh, const
         if (lane + 32 < K) sh.T[lane + 32][c] = v1;
     }
     __syncthreads();
-    for (int e2 = tid; e2 < nF * nc; e2 += PB) {
+    for (int e2 = tid; e2 < nF * nc; e2 += NT) {
         const int q = e2 / nc, c = c0 + e2 % nc;
         float acc = 0.f;
         for (int k = 0; k < K; ++k) acc = fmaf(brow32(P, sh, F, q, k), sh.T[k][c - c0], acc);
@@ -365,14 +384,15 @@ __device__ __noinline__ void woodbury32(const PolDev& P, PolishShared& sh, const
     __syncthreads();
 }
 
-// FP32 solve of Sigma_FF x = r for the columns c0..c1 of Y (in: D^{-1} r; out: x) with the
+// FP32 solve of Sigma_FF x = r for the columns c0..c1 of Y (in: r; out: x) with the
 // Cholesky factor of Sigma_FF itself (|F| <= K, free set in shared memory): one warp per
 // column, rows lane and lane + 32 in registers. Block-collective.
+template <int NT>
 __device__ __noinline__ void direct32(PolishShared& sh, const FreeSet& F, int nF, int c0, int c1) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int c = c0 + warp; c < c1; c += PB / 32) {
-        float v0 = lane < nF ? float(F.Y[(size_t)lane * YS + c] / F.dinv[lane]) : 0.f;
-        float v1 = lane + 32 < nF ? float(F.Y[(size_t)(lane + 32) * YS + c] / F.dinv[lane + 32]) : 0.f;
+    for (int c = c0 + warp; c < c1; c += NT / 32) {
+        float v0 = lane < nF ? float(F.Y[(size_t)lane * YS + c]) : 0.f;
+        float v1 = lane + 32 < nF ? float(F.Y[(size_t)(lane + 32) * YS + c]) : 0.f;
         for (int r = 0; r < nF; ++r) {
             const float x = __shfl_sync(0xffffffffu, r < 32 ? v0 : v1, r & 31) * sh.Ldinv[r];
             if (lane > r && lane < nF) v0 = fmaf(-sh.C[lane][r], x, v0);
@@ -391,21 +411,23 @@ __device__ __noinline__ void direct32(PolishShared& sh, const FreeSet& F, int nF
     __syncthreads();
 }
 
+template <int NT>
 __device__ __forceinline__ void solve32(const PolDev& P, PolishShared& sh, const FreeSet& F, int nF, int c0,
                                         int c1, bool direct) {
-    if (direct) direct32(sh, F, nF, c0, c1);
-    else woodbury32(P, sh, F, nF, c0, c1);
+    if (direct) direct32<NT>(sh, F, nF, c0, c1);
+    else woodbury32<NT>(P, sh, F, nF, c0, c1);
 }
 
 // (b3) of a polish round: the FP32 matrix to factor (Sigma_FF = B_F F B_F' + D_F when
 // ``direct``, else the Woodbury capacitance C = F^{-1} + B_F' D_F^{-1} B_F) and its Cholesky
 // factor in sh.C (lower triangle, diagonal included) with the reciprocal diagonal in sh.Ldinv.
 // Returns false when a pivot is not positive. Block-collective.
+template <int NT>
 __device__ __noinline__ bool factor32(const PolDev& P, PolishShared& sh, const FreeSet& F, int nF, bool direct) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int K = P.K, nS = direct ? nF : K;
     if (direct) {
-        for (int e2 = tid; e2 < nS * nS; e2 += PB) {
+        for (int e2 = tid; e2 < nS * nS; e2 += NT) {
             const int r = e2 / nS, c = e2 % nS;
             if (c > r) continue;
             float acc = (r == c) ? float(P.d64[F.Fl[r]]) : 0.f;
@@ -413,7 +435,7 @@ __device__ __noinline__ bool factor32(const PolDev& P, PolishShared& sh, const F
             sh.C[r][c] = acc;
         }
     } else {
-        for (int e2 = tid; e2 < K * K; e2 += PB) {
+        for (int e2 = tid; e2 < K * K; e2 += NT) {
             const int r = e2 / K, c = e2 % K;
             if (c > r) continue;
             float acc = (r == c) ? 1.f / sh.f32s[r] : 0.f;
@@ -432,21 +454,21 @@ __device__ __noinline__ bool factor32(const PolDev& P, PolishShared& sh, const F
         const float piv = sh.C[c][c];
         if (!(piv > 0.f)) { chol_ok = false; break; }          // every thread reads the same pivot
         const float ip = 1.f / piv;
-        for (int r = c + 1 + warp; r < nS; r += PB / 32) {
+        for (int r = c + 1 + warp; r < nS; r += NT / 32) {
             const float lr = sh.C[r][c] * ip;
             for (int q = c + 1 + lane; q <= r; q += 32) sh.C[r][q] = fmaf(-lr, sh.C[q][c], sh.C[r][q]);
         }
         __syncthreads();
     }
     if (chol_ok) {
-        for (int c = tid; c < nS; c += PB) sh.Ldinv[c] = sqrtf(sh.C[c][c]);
+        for (int c = tid; c < nS; c += NT) sh.Ldinv[c] = sqrtf(sh.C[c][c]);
         __syncthreads();
-        for (int e2 = tid; e2 < nS * nS; e2 += PB) {
+        for (int e2 = tid; e2 < nS * nS; e2 += NT) {
             const int r = e2 / nS, c = e2 % nS;
             if (c < r) sh.C[r][c] /= sh.Ldinv[c];
         }
         __syncthreads();
-        for (int c = tid; c < nS; c += PB) { sh.C[c][c] = sh.Ldinv[c]; sh.Ldinv[c] = 1.f / sh.Ldinv[c]; }
+        for (int c = tid; c < nS; c += NT) { sh.C[c][c] = sh.Ldinv[c]; sh.Ldinv[c] = 1.f / sh.Ldinv[c]; }
     }
     return chol_ok;
 }
@@ -464,12 +486,12 @@ __device__ __noinline__ bool factor32(const PolDev& P, PolishShared& sh, const F
 // so ||w - w*||_2 <= (||r||_2 + sqrt(||r||_2^2 + 4 m C)) / (2 m). This holds for a point
 // that meets the constraints; the primal residuals reported beside it say by how much
 // the returned point misses them (to FP64 rounding for a certified account).
-__device__ __noinline__ double err_bound(const PolDev& P, const PolishShared& sh, double r2, double sw, double tu,
-                                         double tau, double nu, double theta) {
+// (err_terms: a lane's share of the bands' and factor rows' terms, to be summed over the warp.)
+__device__ __forceinline__ void err_terms(const PolDev& P, const PolishShared& sh, double& wrong, double& C) {
     const double m = 2.0 * P.dmin;
-    if (!(m > 0.0)) return INFINITY;
-    double wrong = 0.0, C = fabs(nu) * fabs(sw - 1.0);
-    for (int s = 0; s < P.S; ++s) {
+    const int lane = threadIdx.x & 31;
+    if (!(m > 0.0)) return;
+    for (int s = lane; s < P.S; s += 32) {
         // lambda_s >= 0 prices the upper edge and lambda_s <= 0 the lower one; a multiplier
         // on an infinite edge has no such reading and counts as of the wrong sign
         // Either reading gives a valid bound, so each multiplier takes the one that adds less
@@ -481,14 +503,22 @@ __device__ __noinline__ double err_bound(const PolDev& P, const PolishShared& sh
         if (sqrt(as_comp / m) <= sqrt(double(P.N)) * fabs(ls) / m) C += as_comp;
         else wrong += fabs(ls);
     }
-    for (int k = 0; k < P.K && P.flo; ++k) {
-        // factor rows, read like the bands (kappa_k >= 0 prices the upper bound)
-        const double kk = sh.kap_s[k], hk = sh.t64[k];
-        if (kk == 0.0) continue;
-        const double edge = kk > 0.0 ? sh.fhi_s[k] : sh.flo_s[k];
-        // (a multiplier on an infinite bound has no such reading: C, and the bound, become +inf)
-        C += isfinite(edge) ? fabs(kk) * fabs(edge - hk) : INFINITY;
-    }
+    if (P.flo)
+        for (int k = lane; k < P.K; k += 32) {
+            // factor rows, read like the bands (kappa_k >= 0 prices the upper bound)
+            const double kk = sh.kap_s[k], hk = sh.t64[k];
+            if (kk == 0.0) continue;
+            const double edge = kk > 0.0 ? sh.fhi_s[k] : sh.flo_s[k];
+            // (a multiplier on an infinite bound has no such reading: C, and the bound, become +inf)
+            C += isfinite(edge) ? fabs(kk) * fabs(edge - hk) : INFINITY;
+        }
+}
+
+__device__ __forceinline__ double err_bound(const PolDev& P, double r2, double wrong, double C, double sw, double tu,
+                                            double tau, double nu, double theta) {
+    const double m = 2.0 * P.dmin;
+    if (!(m > 0.0)) return INFINITY;
+    C += fabs(nu) * fabs(sw - 1.0);
     if (theta != 0.0) {
         const double as_comp = (isfinite(tau) && theta > 0.0) ? theta * fabs(tau - tu) : INFINITY;
         if (sqrt(as_comp / m) <= sqrt(double(P.N)) * fabs(theta) / m) C += as_comp;
@@ -498,7 +528,7 @@ __device__ __noinline__ double err_bound(const PolDev& P, const PolishShared& sh
     return (re + sqrt(re * re + 4.0 * m * C)) / (2.0 * m);
 }
 
-// The factor-exposure rows' checks of one account (thread 0), like the bands': a row outside the
+// The factor-exposure rows' checks of one account (a lane's factors), like the bands': a row outside the
 // working set joins it when violated; a working row leaves it when its multiplier has the wrong
 // sign, or, found dependent on the free set, when it holds strictly inside its bounds.
 __device__ __noinline__ void factor_row_checks(const PolDev& P, PolishShared& sh, int a, int m, double tol_p,
@@ -510,13 +540,13 @@ __device__ __noinline__ void factor_row_checks(const PolDev& P, PolishShared& sh
             if (sh.rows[r] == row) return sh.used[r] == 0;
         return false;
     };
-    for (int k = 0; k < K; ++k) {
+    for (int k = threadIdx.x & 31; k < K; k += 32) {
         const double hk = sh.t64[k], hi = sh.fhi_s[k], lo = sh.flo_s[k];
         r_exp = fmax(r_exp, fmax(lo - hk, hk - hi));
         const int wf = sh.wf_s[k];
         const double kk = sh.kap_s[k];
         const bool off = wf != 0 && fabs(hk - (wf > 0 ? hi : lo)) > tol_p;
-        auto set_wf = [&](int v) { sh.wf_s[k] = v; P.wfac[a * K + k] = v; };
+        auto set_wf = [&](int v) { note_change(sh, P.N + SMAX + 1 + k, sh.wf_s[k], v); sh.wf_s[k] = v; P.wfac[a * K + k] = v; };
         if (off && row_dependent(S + 1 + k)) {
             ++bviol;
             if (wf > 0 ? hk < hi : hk > lo) { set_wf(0); ++dep_in; }
@@ -537,7 +567,8 @@ __device__ __noinline__ void factor_row_checks(const PolDev& P, PolishShared& sh
     }
 }
 
-__global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // two blocks per SM
+template <int NT>
+__global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) k_polish(PolDev P, int rounds) {
     const int a = blockIdx.x;
     if ((P.skip && P.skip[a]) || P.done[a] || (P.sel && P.sel[a] != P.gen)) return;
     extern __shared__ unsigned char smem_raw[];
@@ -549,20 +580,21 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
     int* NZl = P.NZlist + (size_t)a * P.FMAX;
     double* W = P.W + base;
     const double tol_d = P.tol_dual, tol_p = P.tol_primal;
-    for (int s2 = tid; s2 < S; s2 += PB) {
+    for (int s2 = tid; s2 < S; s2 += NT) {
         sh.blo_s[s2] = P.band_lo[a * S + s2];
         sh.bhi_s[s2] = P.band_hi[a * S + s2];
         sh.wb_s[s2] = P.wband[a * S + s2];
     }
-    for (int k = tid; k < K; k += PB) {
+    for (int k = tid; k < K; k += NT) {
         sh.wf_s[k] = P.wfac ? P.wfac[a * K + k] : 0;
         sh.flo_s[k] = P.flo ? P.flo[a * K + k] : -INFINITY;
         sh.fhi_s[k] = P.fhi ? P.fhi[a * K + k] : INFINITY;
     }
+    if (tid == 0) sh.hash = 0;
     __syncthreads();
     for (int round = 0; round < rounds; ++round) {
         // ---- (a) ordered compaction in coalesced warp tiles; W of the fixed entries
-        const int Lw = cdiv(cdiv(N, PB / 32), 32) * 32;
+        const int Lw = cdiv(cdiv(N, NT / 32), 32) * 32;
         const int w0r = min(N, warp * Lw), w1r = min(N, w0r + Lw);
         int nf = 0, nn = 0;
         double sa = 0.0, ca = 0.0, ta = 0.0, oa = 0.0;
@@ -625,7 +657,7 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
         if (tid == 0) {
             int of = 0, on = 0;
             double ss = 0.0, cc = 0.0, tt = 0.0, oo = 0.0;
-            for (int t = 0; t < PB / 32; ++t) {
+            for (int t = 0; t < NT / 32; ++t) {
                 const int f = sh.cntF[t], n = sh.cntN[t];
                 sh.cntF[t] = of; sh.cntN[t] = on;
                 of += f; on += n;
@@ -678,13 +710,17 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
         const double sumA = sh.sumA[0], capA = sh.capA[0], turnA = sh.turnA[0], objA = sh.objA[0];
         // ---- (b1) h_A = B' w_A (FP64) over the nonzero fixed entries
         {
-            const int k = tid >> 2, sub = tid & 3;
+            constexpr int L = NT / KMAX;
+            const int k = tid / L, sub = tid % L;
             double acc = 0.0;
-            if (k < K)
-                for (int q = sub; q < nNZ; q += 4) {
+            if (k < K) {
+#pragma unroll 4
+                for (int q = sub; q < nNZ; q += L) {
                     const int p = NZl[q];
                     acc += W[p] * P.B64[(size_t)p * K + k];
                 }
+            }
+            if (L == 8) acc += __shfl_xor_sync(0xffffffffu, acc, 4);
             acc += __shfl_xor_sync(0xffffffffu, acc, 2);
             acc += __shfl_xor_sync(0xffffffffu, acc, 1);
             if (sub == 0 && k < K) {
@@ -694,7 +730,7 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
         }
         // per sector, the sum of the fixed weights (one warp per sector); the sectors of the
         // free entries whose data live in shared memory
-        for (int s2 = warp; s2 < S; s2 += PB / 32) {
+        for (int s2 = warp; s2 < S; s2 += NT / 32) {
             double acc = 0.0;
             for (int q = lane; q < nNZ; q += 32) {
                 const int p = NZl[q];
@@ -703,22 +739,22 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
             acc = warp_sum(acc);
             if (lane == 0) sh.fixS[s2] = acc;
         }
-        for (int q = tid; q < min(nF, FS); q += PB) sh.secF[q] = P.sector[Flg[q]];
+        for (int q = tid; q < min(nF, FS); q += NT) sh.secF[q] = P.sector[Flg[q]];
         __syncthreads();
         // ---- (b2) the free set: shared memory when small; rows of B in FP32 and FP64
         FreeSet F;
         F.in_smem = nF <= FS;
         if (F.in_smem) {
             F.Fl = sh.Fl_s; F.Y = &sh.Ys[0][0]; F.dinv = sh.dinv_s; F.sig = sh.sig_s;
-            for (int q = tid; q < nF; q += PB) sh.Fl_s[q] = Flg[q];
+            for (int q = tid; q < nF; q += NT) sh.Fl_s[q] = Flg[q];
         } else {
             F.Fl = Flg;
             F.Y = P.Y + (size_t)a * P.FMAX * YS;
             F.dinv = P.Fdinv + (size_t)a * P.FMAX;
             F.sig = P.Fsig + (size_t)a * P.FMAX;
         }
-        for (int k = tid; k < K; k += PB) sh.f32s[k] = float(P.f64[k]);
-        for (int e2 = tid; e2 < min(nF, FS) * K; e2 += PB) {
+        for (int k = tid; k < K; k += NT) { sh.f64s[k] = P.f64[k]; sh.f32s[k] = float(P.f64[k]); }
+        for (int e2 = tid; e2 < min(nF, FS) * K; e2 += NT) {
             const int q = e2 / K, k = e2 % K;
             const double b = P.B64[(size_t)Flg[q] * K + k];
             sh.Bd[q][k] = b;
@@ -726,7 +762,7 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
         }
         __syncthreads();
         // g0 (FP64), 1/d, cap signs
-        rows_dot64(P, sh, F, nF, sh.fhA, [&](int q, double bf) {
+        rows_dot64<NT>(P, sh, F, nF, sh.fhA, [&](int q, double bf) {
             const int p = F.Fl[q];
             const size_t e = base + p;
             Pieces pc;
@@ -735,7 +771,9 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
             double* Yq = F.Y + (size_t)q * YS;
             Yq[0] = mu_at(P, e, p) - pc.sl[seg] - 2.0 * bf;
             Yq[COL_W] = 0.0;
-            F.dinv[q] = 1.0 / P.d64[p];
+            const double dq = P.d64[p];
+            F.dinv[q] = 1.0 / dq;
+            if (q < FS) sh.d_s[q] = dq;
             if (q < FS) sh.dinvf_s[q] = float(F.dinv[q]);
             F.sig[q] = seg_sign(pc, seg);
         });
@@ -744,26 +782,27 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
         // set is no larger than K (it then lives in shared memory), else the Woodbury
         // capacitance C = F^{-1} + B_F' D_F^{-1} B_F; then its Cholesky factor
         const bool direct = nF <= K && nF <= FS;
-        const bool chol_ok = factor32(P, sh, F, nF, direct);
+        const bool chol_ok = factor32<NT>(P, sh, F, nF, direct);
         __syncthreads();
         if (!chol_ok) {
             if (tid == 0) P.done[a] = 2;
             return;
         }
         // ---- (b4) Y_E = Sigma_FF^{-1} E_F' (FP32, stored in Y columns 1..m)
-        for (int e2 = tid; e2 < nF * m; e2 += PB) {
+        for (int e2 = tid; e2 < nF * m; e2 += NT) {
             const int q = e2 / m, r = e2 % m;
-            F.Y[(size_t)q * YS + 1 + r] = coef_q(P, sh, F, sh.rows[r], q) * F.dinv[q];
+            const double cf = coef_q(P, sh, F, sh.rows[r], q);
+            F.Y[(size_t)q * YS + 1 + r] = direct ? cf : cf * F.dinv[q];
         }
         __syncthreads();
-        solve32(P, sh, F, nF, 1, 1 + m, direct);
+        solve32<NT>(P, sh, F, nF, 1, 1 + m, direct);
         // Schur matrix S = 1/2 E Y_E, and row edges e = edge - fixed part
-        for (int e2 = warp; e2 < m * m; e2 += PB / 32) {
+        for (int e2 = warp; e2 < m * m; e2 += NT / 32) {
             const int r = e2 / m, c = e2 % m;
             const double acc = erow_dot(P, sh, F, nF, sh.rows[r], 1 + c, lane);
             if (lane == 0) sh.Sf[r][c] = 0.5 * acc;
         }
-        for (int r = tid; r < m; r += PB) {
+        for (int r = tid; r < m; r += NT) {
             const int row = sh.rows[r];
             double e_r;
             if (row < 0) {
@@ -798,15 +837,22 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
                 if (p < 0 || !(fabs(sh.Sf[p][p]) > 1e-9 * scale)) break;
                 sh.used[p] = 1;
                 sh.order[nc++] = p;
+                sh.ipiv[p] = 1.0 / sh.Sf[p][p];
                 for (int j = 0; j < m; ++j) {
                     if (sh.used[j]) continue;
-                    const double f = sh.Sf[j][p] / sh.Sf[p][p];
+                    const double f = sh.Sf[j][p] * sh.ipiv[p];
                     // only columns not yet pivoted: pivoted ones of row j hold its multipliers
                     for (int q = 0; q < m; ++q) if (!sh.used[q]) sh.Sf[j][q] -= f * sh.Sf[p][q];
                     sh.Sf[j][p] = f;                       // multiplier of row j against pivot p
                 }
             }
             sh.nc = nc;
+            // A cap that depends on the budget (every free weight on one side of its holding) keeps the
+            // iterations' multiplier: the budget's takes up the difference on the free weights, while
+            // with theta = 0 nearly every held name would seem to want to move
+            if (P.theta_hint)
+                for (int r = 1; r < m; ++r)
+                    if (!sh.used[r] && sh.rows[r] == S) sh.lam[r] = fmax(double(P.theta_hint[a]), 0.0);
             sh.fail = (nc == 0);
         }
         __syncthreads();
@@ -817,43 +863,53 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
         const int ndep = m - sh.nc;
         // ---- (b5) iterative refinement: FP64 residuals, FP32 corrections
         for (int it = 0; it < IR_STEPS; ++it) {
-            // t = B_F' w_F (FP64)
-            cols_dot64(P, sh, F, nF, [&](int q) { return F.Y[(size_t)q * YS + COL_W]; },
-                       [&](int k, double acc) { sh.t64[k] = P.f64[k] * acc; });
+            // t = B_F' w_F (FP64); the first step starts from w = 0, lam = 0
+            if (it > 0) cols_dot64<NT>(P, sh, F, nF, [&](int q) { return F.Y[(size_t)q * YS + COL_W]; },
+                       [&](int k, double acc) { sh.t64[k] = sh.f64s[k] * acc; });
             __syncthreads();
-            // r1 = g0 - 2 Sigma_FF w - E' lam ; stored scaled by D^{-1} in COL_R
+            // r1 = g0 - 2 Sigma_FF w - E' lam ; stored (scaled by D^{-1} for the Woodbury form) in COL_R
             double rmax = 0.0;
-            rows_dot64(P, sh, F, nF, sh.t64, [&](int q, double bt) {
-                const int p = F.Fl[q];
-                double* Yq = F.Y + (size_t)q * YS;
-                double r1 = Yq[0] - 2.0 * (bt + P.d64[p] * Yq[COL_W]);
-                for (int r = 0; r < m; ++r) r1 -= coef_q(P, sh, F, sh.rows[r], q) * sh.lam[r];
-                rmax = fmax(rmax, fabs(r1));
-                Yq[COL_R] = r1 * F.dinv[q];
-            });
-            // r2 = e - E w
-            for (int r = warp; r < m; r += PB / 32) {
-                const double acc = erow_dot(P, sh, F, nF, sh.rows[r], COL_W, lane);
-                if (lane == 0) sh.rr2[r] = sh.erhs[r] - acc;
+            if (it == 0) {
+                for (int q = tid; q < nF; q += NT) {
+                    double* Yq = F.Y + (size_t)q * YS;
+                    rmax = fmax(rmax, fabs(Yq[0]));
+                    Yq[COL_R] = direct ? Yq[0] : Yq[0] * F.dinv[q];
+                }
+                for (int r = tid; r < m; r += NT) sh.rr2[r] = sh.erhs[r];
+            } else {
+                rows_dot64<NT>(P, sh, F, nF, sh.t64, [&](int q, double bt) {
+                    double* Yq = F.Y + (size_t)q * YS;
+                    double r1 = Yq[0] - 2.0 * (bt + (q < FS ? sh.d_s[q] : P.d64[F.Fl[q]]) * Yq[COL_W]);
+                    for (int r = 0; r < m; ++r) r1 -= coef_q(P, sh, F, sh.rows[r], q) * sh.lam[r];
+                    rmax = fmax(rmax, fabs(r1));
+                    Yq[COL_R] = direct ? r1 : r1 * F.dinv[q];
+                });
+                // r2 = e - E w
+                for (int r = warp; r < m; r += NT / 32) {
+                    const double acc = erow_dot(P, sh, F, nF, sh.rows[r], COL_W, lane);
+                    if (lane == 0) sh.rr2[r] = sh.erhs[r] - acc;
+                }
             }
             rmax = warp_max(rmax);
             if (lane == 0) sh.red[warp][0] = rmax;
             __syncthreads();
             // converged: every warp's residual maximum and every row residual within its limit,
             // tested lane-wise in each warp (the same answer in every warp; a NaN never passes)
-            bool conv = lane >= PB / 32 || sh.red[lane][0] <= 1e-15;
+            bool conv = lane >= NT / 32 || sh.red[lane][0] <= 1e-15;
             for (int r = lane; r < m; r += 32) conv = conv && fabs(sh.rr2[r]) <= 1e-16;
             conv = __all_sync(0xffffffffu, conv);
             if (it > 0 && conv) break;
             // Yr = Sigma_FF^{-1} r1 (FP32)
-            solve32(P, sh, F, nF, COL_R, COL_R + 1, direct);
+            solve32<NT>(P, sh, F, nF, COL_R, COL_R + 1, direct);
             // dlam = S^{-1} (1/2 E Yr - r2) with the eliminated S
-            for (int r = warp; r < m; r += PB / 32) {
+            for (int r = warp; r < m; r += NT / 32) {
                 const double acc = erow_dot(P, sh, F, nF, sh.rows[r], COL_R, lane);
                 if (lane == 0) sh.dlam[r] = 0.5 * acc - sh.rr2[r];
             }
             __syncthreads();
-            if (tid == 0) {
+            if (m == 1) {
+                if (tid == 0) { sh.dlam[0] *= sh.ipiv[0]; sh.lam[0] += sh.dlam[0]; }
+            } else if (tid == 0) {
                 // forward: apply the recorded eliminations in pivot order
                 for (int k = 0; k < sh.nc; ++k) {
                     const int p = sh.order[k];
@@ -863,19 +919,19 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
                         if (later && j != p) sh.dlam[j] -= sh.Sf[j][p] * sh.dlam[p];
                     }
                 }
-                double x[PMAXROWS];
+                double* x = sh.xrow;
                 for (int r = 0; r < m; ++r) x[r] = 0.0;
                 for (int k = sh.nc - 1; k >= 0; --k) {
                     const int p = sh.order[k];
                     double v = sh.dlam[p];
                     for (int kk = k + 1; kk < sh.nc; ++kk) { const int q = sh.order[kk]; v -= sh.Sf[p][q] * x[q]; }
-                    x[p] = v / sh.Sf[p][p];
+                    x[p] = v * sh.ipiv[p];
                 }
                 for (int r = 0; r < m; ++r) { sh.dlam[r] = x[r]; sh.lam[r] += x[r]; }
             }
             __syncthreads();
             // dw = 1/2 (Yr - Y_E dlam)
-            for (int q = tid; q < nF; q += PB) {
+            for (int q = tid; q < nF; q += NT) {
                 double* Yq = F.Y + (size_t)q * YS;
                 double acc = Yq[COL_R];
                 for (int r = 0; r < m; ++r) acc -= Yq[1 + r] * sh.dlam[r];
@@ -884,17 +940,17 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
             __syncthreads();
         }
         // ---- (b6) the solved point: W_F, h = h_A + B_F' w_F, multipliers
-        for (int q = tid; q < nF; q += PB) W[F.Fl[q]] = F.Y[(size_t)q * YS + COL_W];
-        cols_dot64(P, sh, F, nF, [&](int q) { return F.Y[(size_t)q * YS + COL_W]; }, [&](int k, double bw) {
+        for (int q = tid; q < nF; q += NT) W[F.Fl[q]] = F.Y[(size_t)q * YS + COL_W];
+        cols_dot64<NT>(P, sh, F, nF, [&](int q) { return F.Y[(size_t)q * YS + COL_W]; }, [&](int k, double bw) {
             const double acc = sh.hA[k] + bw;
             const double fhk = P.f64[k] * acc;
             sh.t64[k] = acc;
             sh.fh[k] = fhk;
             sh.fh32[k] = float(fhk);
         });
-        for (int k = K + tid; k < KMAX; k += PB) sh.fh32[k] = 0.f;
-        for (int s2 = tid; s2 < S; s2 += PB) sh.lam_s[s2] = 0.0;
-        for (int k = tid; k < K; k += PB) sh.kap_s[k] = 0.0;
+        for (int k = K + tid; k < KMAX; k += NT) sh.fh32[k] = 0.f;
+        for (int s2 = tid; s2 < S; s2 += NT) sh.lam_s[s2] = 0.0;
+        for (int k = tid; k < K; k += NT) sh.kap_s[k] = 0.0;
         __syncthreads();
         double theta = 0.0;
         for (int r = 1; r < m; ++r) if (sh.rows[r] == S) theta = sh.lam[r];
@@ -934,6 +990,10 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
         int nviol = 0;
         double my_margin = INFINITY;
         int my_who = 0;
+        auto set_state = [&](int p, int was, int is) {
+            P.st[base + p] = (int8_t)is;
+            note_change(sh, p, was, is);
+        };
         // FP64 checks of one entry (run 32 entries at a time from the warp's queue); gx, when
         // given, is the entry's exact product B_p . fh computed beforehand
         auto check_entry3 = [&](int p, float g32, const double* gx) {
@@ -974,8 +1034,8 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
                 const double res = fabs(rr + pc.sl[seg] + theta * seg_sign(pc, seg));
                 r_stat = fmax(r_stat, res);
                 r_sq += res * res;
-                if (wv > pc.bp[seg + 1] + tol_p) { ++nviol; P.st[e] = (int8_t)(seg + 1); }
-                else if (wv < pc.bp[seg] - tol_p) { ++nviol; P.st[e] = (int8_t)seg; }
+                if (wv > pc.bp[seg + 1] + tol_p) { ++nviol; set_state(p, code, seg + 1); }
+                else if (wv < pc.bp[seg] - tol_p) { ++nviol; set_state(p, code, seg); }
             } else {
                 const int j = code;
                 const double left = (j > 0) ? pc.sl[j - 1] + theta * seg_sign(pc, j - 1) : -INFINITY;
@@ -994,16 +1054,16 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
                     if (isfinite(right) && -up < my_margin) { my_margin = -up; my_who = p + 1; }
                     if (isfinite(left) && -dn < my_margin) { my_margin = -dn; my_who = -(p + 1); }
                 }
-                if (up > tol_d) { ++nviol; P.st[e] = (int8_t)(ST_FREE + j); }
-                else if (dn > tol_d) { ++nviol; P.st[e] = (int8_t)(ST_FREE + j - 1); }
+                if (up > tol_d) { ++nviol; set_state(p, code, ST_FREE + j); }
+                else if (dn > tol_d) { ++nviol; set_state(p, code, ST_FREE + j - 1); }
             }
         };
         auto check_entry = [&](int p, float g32) { check_entry3(p, g32, nullptr); };
         // the free entries of a free set in shared memory are checked in a pass of their own,
         // with their exact products computed here by the whole block
         const bool free_pass = F.in_smem;
-        if (free_pass) rows_dot64(P, sh, F, nF, sh.fh, [&](int q, double v) { sh.gF[q] = v; });
-        for (int s2 = tid; s2 < S; s2 += PB) sh.lam_s32[s2] = float(sh.lam_s[s2]);
+        if (free_pass) rows_dot64<NT>(P, sh, F, nF, sh.fh, [&](int q, double v) { sh.gF[q] = v; });
+        for (int s2 = tid; s2 < S; s2 += NT) sh.lam_s32[s2] = float(sh.lam_s[s2]);
         __syncthreads();
         float fmargin = INFINITY;
         int fwho = 0;
@@ -1027,8 +1087,8 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
         };
         TileIn cur{}, nxt{};
         if (warp < ntiles) load_tile(warp, cur);
-        for (int ti = warp; ti < ntiles; ti += PB / 32) {
-            if (ti + PB / 32 < ntiles) load_tile(ti + PB / 32, nxt);
+        for (int ti = warp; ti < ntiles; ti += NT / 32) {
+            if (ti + NT / 32 < ntiles) load_tile(ti + NT / 32, nxt);
             const int p = ti * 32 + lane;                 // entries of padding (p >= N) are skipped below
             const int code = cur.code, pwv = cur.pw, sec = cur.sec;
             const float w0v = cur.w0, lov = cur.lo, upv = cur.up, cv = cur.c;
@@ -1038,21 +1098,33 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
             float g32 = 0.f;
             const float* Bt = P.B32p + (size_t)ti * 32 * KMAX;
 #pragma unroll
-            for (int grp = 0; grp < 4; ++grp) {
-                const float4* Br = reinterpret_cast<const float4*>(Bt + (size_t)(grp * 8 + (lane >> 2)) * KMAX) + (lane & 3);
-                float acc = 0.f;
+            for (int half = 0; half < 2; ++half) {
+                // two groups of eight rows at a time, all their loads first; the columns past K are zero
+                // and not read
+                float4 b[2][4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float4 b = __ldg(Br + 4 * i);
-                    acc = fmaf(b.x, fr[i].x, acc);
-                    acc = fmaf(b.y, fr[i].y, acc);
-                    acc = fmaf(b.z, fr[i].z, acc);
-                    acc = fmaf(b.w, fr[i].w, acc);
+                for (int g = 0; g < 2; ++g) {
+                    const float4* Br = reinterpret_cast<const float4*>(Bt + (size_t)((2 * half + g) * 8 + (lane >> 2)) * KMAX) + (lane & 3);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (16 * i < K) b[g][i] = __ldg(Br + 4 * i);
                 }
-                acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-                acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-                const float v = __shfl_sync(0xffffffffu, acc, 4 * (lane & 7));
-                if ((lane >> 3) == grp) g32 = v;
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    float acc = 0.f;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if (16 * i >= K) break;
+                        acc = fmaf(b[g][i].x, fr[i].x, acc);
+                        acc = fmaf(b[g][i].y, fr[i].y, acc);
+                        acc = fmaf(b[g][i].z, fr[i].z, acc);
+                        acc = fmaf(b[g][i].w, fr[i].w, acc);
+                    }
+                    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+                    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+                    const float v = __shfl_sync(0xffffffffu, acc, 4 * (lane & 7));
+                    if ((lane >> 3) == 2 * half + g) g32 = v;
+                }
             }
             bool need = p < N;
             if (need && pwv < 0 && code == 0 && lov == 0.f && upv > 0.f) {
@@ -1080,7 +1152,7 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
         }
         wq.drain(true, lane, check_entry);
         if (free_pass)
-            for (int q = tid; q < nF; q += PB) check_entry3(F.Fl[q], 0.f, &sh.gF[q]);
+            for (int q = tid; q < nF; q += NT) check_entry3(F.Fl[q], 0.f, &sh.gF[q]);
         if (double(fmargin) < my_margin) { my_margin = double(fmargin); my_who = fwho; }
         r_stat = warp_max(r_stat); r_box = warp_max(r_box); r_sq = warp_sum(r_sq);
         obj_lin = warp_sum(obj_lin); sum_w = warp_sum(sum_w); turn = warp_sum(turn);
@@ -1097,7 +1169,7 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
             sh.mmin[warp] = my_margin; sh.mwho[warp] = my_who;
         }
         // sector sums over the entries of nonzero weight: the nonzero fixed and the free ones
-        for (int s2 = warp; s2 < S; s2 += PB / 32) {
+        for (int s2 = warp; s2 < S; s2 += NT / 32) {
             double acc = 0.0;
             for (int q = lane; q < nF; q += 32)
                 if ((q < FS ? sh.secF[q] : P.sector[F.Fl[q]]) == s2) acc += F.Y[(size_t)q * YS + COL_W];
@@ -1105,9 +1177,10 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
             if (lane == 0) sh.secsum[s2] = sh.fixS[s2] + acc;
         }
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0) {
+            // the decisions, a lane per sector (and per factor); sums and maxima over the warp
             double rs = 0, rb = 0, ol = 0, sw = 0, tu = 0, nv = 0, rq = 0;
-            for (int w = 0; w < PB / 32; ++w) {
+            for (int w = 0; w < NT / 32; ++w) {
                 rs = fmax(rs, sh.red[w][0]); rb = fmax(rb, sh.red[w][1]); ol += sh.red[w][2];
                 sw += sh.red[w][3]; tu += sh.red[w][4]; nv += sh.red[w][5]; rq += sh.red[w][6];
             }
@@ -1117,13 +1190,13 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
             double r_exp = 0.0, r_comp = 0.0;
             int bviol = 0, dep_in = 0, dep_out = 0;
             // a working row is dependent when the pivoted elimination left it unpivoted
-            auto set_wb = [&](int s2, int v) { sh.wb_s[s2] = v; P.wband[a * S + s2] = v; };
+            auto set_wb = [&](int s2, int v) { note_change(sh, N + s2, sh.wb_s[s2], v); sh.wb_s[s2] = v; P.wband[a * S + s2] = v; };
             auto row_dependent = [&](int row) {
                 for (int r = 1; r < m; ++r)
                     if (sh.rows[r] == row) return sh.used[r] == 0;
                 return false;
             };
-            for (int s2 = 0; s2 < S; ++s2) {
+            for (int s2 = lane; s2 < S; s2 += 32) {
                 const double ssum = sh.secsum[s2];
                 const double hi = sh.bhi_s[s2], lo = sh.blo_s[s2];
                 r_exp = fmax(r_exp, fmax(lo - ssum, ssum - hi));
@@ -1152,58 +1225,70 @@ __global__ void __launch_bounds__(PB, 2) k_polish(PolDev P, int rounds) {   // t
                     }
                 }
             }
-            double r_turn = 0.0;
-            const double tau = P.tau[a];
-            if (isfinite(tau)) {
-                r_turn = fmax(tu - tau, 0.0);
-                if (!P.wcap[a]) {
-                    if (tu > tau + tol_p) { ++bviol; P.wcap[a] = 1; }
-                } else {
-                    const bool off = fabs(tu - tau) > tol_p;
-                    if (off && row_dependent(S)) {
-                        ++bviol;
-                        if (tu < tau) { P.wcap[a] = 0; ++dep_in; }
-                        else ++dep_out;
-                    } else if (off) {
-                        ++bviol;
-                    }
-                    r_comp = fmax(r_comp, fabs(theta) * fabs(tau - tu));
-                    if (theta < -tol_d) { ++bviol; r_comp = fmax(r_comp, -theta); P.wcap[a] = 0; }
-                }
-            }
             // factor rows: exposures h = B'w against their bounds, like the bands
             if (P.flo) factor_row_checks(P, sh, a, m, tol_p, tol_d, r_exp, r_comp, bviol, dep_in, dep_out);
-            const double r_budget = fabs(sw - 1.0);
-            if (r_budget > tol_p) ++bviol;
-            const int total = int(nv) + bviol;
-            if (dep_out > 0 || (total > 0 && ndep > 0 && dep_in == 0)) {
-                // a working row is dependent on the free set and cannot be met by it: free the
-                // fixed entry closest to leaving its breakpoint, in the direction of least resistance
-                double bm = INFINITY;
-                int who = 0;
-                for (int w = 0; w < PB / 32; ++w)
-                    if (sh.mmin[w] < bm || (sh.mmin[w] == bm && abs(sh.mwho[w]) < abs(who))) { bm = sh.mmin[w]; who = sh.mwho[w]; }
-                if (who != 0) {
-                    const size_t e = base + (abs(who) - 1);
-                    const int j = P.st[e];
-                    if (j < ST_FREE) P.st[e] = (int8_t)(who > 0 ? ST_FREE + j : ST_FREE + j - 1);
+            double wrong = 0.0, slack = 0.0;
+            err_terms(P, sh, wrong, slack);
+            for (int s2 = lane; s2 < S; s2 += 32) P.lam[a * S + s2] = sh.lam_s[s2];
+            if (P.kappa) for (int k = lane; k < K; k += 32) P.kappa[a * K + k] = sh.kap_s[k];
+            r_exp = warp_max(r_exp); r_comp = warp_max(r_comp);
+            wrong = warp_sum(wrong); slack = warp_sum(slack);
+            bviol = warp_sum(bviol); dep_in = warp_sum(dep_in); dep_out = warp_sum(dep_out);
+            if (lane == 0) {
+                double r_turn = 0.0;
+                const double tau = P.tau[a];
+                if (isfinite(tau)) {
+                    r_turn = fmax(tu - tau, 0.0);
+                    if (!P.wcap[a]) {
+                        if (tu > tau + tol_p) { ++bviol; P.wcap[a] = 1; note_change(sh, N + SMAX, 0, 1); }
+                    } else {
+                        const bool off = fabs(tu - tau) > tol_p;
+                        if (off && row_dependent(S)) {
+                            ++bviol;
+                            if (tu < tau) { P.wcap[a] = 0; note_change(sh, N + SMAX, 1, 0); ++dep_in; }
+                            else ++dep_out;
+                        } else if (off) {
+                            ++bviol;
+                        }
+                        r_comp = fmax(r_comp, fabs(theta) * fabs(tau - tu));
+                        if (theta < -tol_d) { ++bviol; r_comp = fmax(r_comp, -theta); if (P.wcap[a]) note_change(sh, N + SMAX, 1, 0); P.wcap[a] = 0; }
+                    }
                 }
+                const double r_budget = fabs(sw - 1.0);
+                if (r_budget > tol_p) ++bviol;
+                const int total = int(nv) + bviol;
+                if (dep_out > 0 || (total > 0 && ndep > 0 && dep_in == 0)) {
+                    // a working row is dependent on the free set and cannot be met by it: free the
+                    // fixed entry closest to leaving its breakpoint, in the direction of least resistance
+                    double bm = INFINITY;
+                    int who = 0;
+                    for (int w = 0; w < NT / 32; ++w)
+                        if (sh.mmin[w] < bm || (sh.mmin[w] == bm && abs(sh.mwho[w]) < abs(who))) { bm = sh.mmin[w]; who = sh.mwho[w]; }
+                    if (who != 0) {
+                        const size_t e = base + (abs(who) - 1);
+                        const int j = P.st[e];
+                        if (j < ST_FREE) set_state(abs(who) - 1, j, who > 0 ? ST_FREE + j : ST_FREE + j - 1);
+                    }
+                }
+                double* dg = P.diag + (size_t)a * PRISM_NDIAG;
+                dg[PRISM_DIAG_BUDGET] = r_budget;
+                dg[PRISM_DIAG_BOX] = fmax(rb, 0.0);
+                dg[PRISM_DIAG_EXPOSURE] = fmax(r_exp, 0.0);
+                dg[PRISM_DIAG_TURNOVER] = r_turn;
+                dg[PRISM_DIAG_STAT] = rs;
+                dg[PRISM_DIAG_COMP] = r_comp;
+                dg[PRISM_DIAG_OBJ] = quad + ol;
+                dg[PRISM_DIAG_ERR_EST] = err_bound(P, sqrt(rq), wrong, slack, sw, tu, tau, nu, theta);
+                P.nu[a] = nu;
+                P.theta[a] = theta;
+                if (total == 0) P.done[a] = 1;
+                // A set met before: the rounds repeat themselves, so that the account has nothing to gain from
+                // the rest of them (it goes back to the iterations, unless there is no going back)
+                bool again = false;
+                for (int r = 0; r < min(round, 8); ++r) again |= sh.past[r] == sh.hash;
+                sh.past[round & 7] = sh.hash;
+                sh.go = total > 0 && !(again && P.retry);
             }
-            double* dg = P.diag + (size_t)a * PRISM_NDIAG;
-            dg[PRISM_DIAG_BUDGET] = r_budget;
-            dg[PRISM_DIAG_BOX] = fmax(rb, 0.0);
-            dg[PRISM_DIAG_EXPOSURE] = fmax(r_exp, 0.0);
-            dg[PRISM_DIAG_TURNOVER] = r_turn;
-            dg[PRISM_DIAG_STAT] = rs;
-            dg[PRISM_DIAG_COMP] = r_comp;
-            dg[PRISM_DIAG_OBJ] = quad + ol;
-            dg[PRISM_DIAG_ERR_EST] = err_bound(P, sh, sqrt(rq), sw, tu, tau, nu, theta);
-            P.nu[a] = nu;
-            P.theta[a] = theta;
-            for (int s2 = 0; s2 < S; ++s2) P.lam[a * S + s2] = sh.lam_s[s2];
-            if (P.kappa) for (int k = 0; k < K; ++k) P.kappa[a * K + k] = sh.kap_s[k];
-            if (total == 0) P.done[a] = 1;
-            sh.go = (total > 0);
         }
         __syncthreads();
         if (!sh.go) break;
@@ -1308,10 +1393,20 @@ size_t polish_smem_bytes() { return sizeof(PolishShared); }
 
 void launch_classify(const PolDev& P, cudaStream_t st) { k_classify<<<P.M, PB, 0, st>>>(P); }
 
-// Up to `rounds` active-set rounds for every account not yet settled, in one launch.
+// Up to `rounds` active-set rounds for every account not yet settled, in one launch: blocks of 256 threads,
+// two to an SM, or of 512 when there are no more accounts than SMs (the passes over all entries then
+// take half the time).
 void launch_polish(const PolDev& P, int rounds, cudaStream_t st) {
-    cudaFuncSetAttribute(k_polish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PolishShared));
-    k_polish<<<P.M, PB, sizeof(PolishShared), st>>>(P, rounds);
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (P.M <= sms) {
+        cudaFuncSetAttribute(k_polish<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PolishShared));
+        k_polish<512><<<P.M, 512, sizeof(PolishShared), st>>>(P, rounds);
+    } else {
+        cudaFuncSetAttribute(k_polish<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PolishShared));
+        k_polish<256><<<P.M, 256, sizeof(PolishShared), st>>>(P, rounds);
+    }
 }
 
 void launch_fallback(const PolDev& P, cudaStream_t st) {

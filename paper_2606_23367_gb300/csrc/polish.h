@@ -48,9 +48,11 @@ struct PolDev {
     const float* eta_hi_f = nullptr;    // M x S
     const float* eta_lo_f = nullptr;
     const float* theta_f = nullptr;     // M
+    const float* theta_hint = nullptr;  // M, or null: the cap multiplier of the iterations
     int* skip = nullptr;                // M: 1 = leave this account alone
     const int* sel = nullptr;           // M: when set, only the accounts with sel[a] == gen
     int gen = 0;
+    int retry = 0;                      // 1: an account left unsettled goes back to the iterations
     // state and scratch
     int8_t* st = nullptr;               // M x Npad entry state
     int* wband = nullptr;               // M x S working bands
