@@ -83,6 +83,8 @@ struct SolveCache {
     char* arena = nullptr;
     size_t arena_bytes = 0;
     int* pinned = nullptr;          // host-pinned counter readback
+    static constexpr size_t BOX = 256 * 1024;
+    char* box = nullptr;            // pinned, 2 x BOX: small host inputs on their way in, small outputs back
     cudaGraphExec_t gexec = nullptr;
     Dev gdev;                       // Dev the graph was captured with
     bool have_graph = false;
@@ -118,7 +120,7 @@ void release_cache(prism_universe* uh);
 // ---------------------------------------------------------------------------
 enum : int { ERR_INDEX = 1, ERR_NONFINITE = 2, ERR_BOUNDS = 4, ERR_DUP = 8, ERR_COST = 16, ERR_LEN = 32,
               ERR_LOT_OFFSETS = 64, ERR_LOT_COUNT = 128, ERR_LOT_LOWER = 256, ERR_LOT_DATA = 512, ERR_LOT_SUM = 1024,
-              ERR_BENCH = 2048, ERR_TILT = 4096 };
+              ERR_BENCH = 2048, ERR_TILT = 4096, ERR_BAND = 8192, ERR_CAP = 16384 };
 
 struct PackArgs {
     int M, N, Npad;
@@ -128,7 +130,7 @@ struct PackArgs {
     const int* inv_perm;
     double *W0, *LO, *UP, *C;
     float *W0f, *LOf, *UPf, *Cf;
-    int* member;
+    int* member;                 // ragged books: 1 at the account's positions; else null
     int* err;
     int64_t nnz;
 };
@@ -158,11 +160,78 @@ __global__ void k_pack(PackArgs A) {
     const size_t d = (size_t)a * A.Npad + A.inv_perm[i];
     if (A.asset_idx) {
         if (atomicExch(&A.member[d], 1) != 0) { atomicOr(A.err, ERR_DUP); return; }
-    } else {
-        A.member[d] = 1;                   // position i of account a: no duplicate is possible
-    }
+    }                                      // (else position i of account a: no duplicate is possible)
     A.W0[d] = w0; A.LO[d] = l; A.UP[d] = u; A.C[d] = c;
     A.W0f[d] = float(w0); A.LOf[d] = float(l); A.UPf[d] = float(u); A.Cf[d] = float(c);
+}
+
+// Everything a solve starts from per account, in one launch, where some 35 memsets and small copies
+// stood (each 2-3 us on the stream: 0.12 of the 0.5 ms of a one-account call): bands, caps and factor
+// bounds checked and in FP32 too, and the state of the iterations and the polish.
+struct SetupArgs {
+    int M, S, K, rho_idx, n_ctr;
+    const double *band_lo, *band_hi, *tau, *flo, *fhi;     // device; tau, flo and fhi may be null
+    double *bd_lo, *bd_hi, *bd_tau, *bd_flo, *bd_fhi;
+    float *bd_lof, *bd_hif, *bd_tauf, *bd_flof, *bd_fhif;
+    Dev D;
+    PolDev P;
+    int* err;                                              // [0] flags, [2] some cap is finite
+};
+
+__global__ void k_setup(SetupArgs A) {
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const Dev& D = A.D;
+    const PolDev& P = A.P;
+    if (e < (int64_t)A.M * A.S) {
+        const double lo = A.band_lo[e], hi = A.band_hi[e];
+        if (isnan(lo) || isnan(hi) || lo > hi) atomicOr(A.err, ERR_BAND);
+        A.bd_lo[e] = lo; A.bd_hi[e] = hi;
+        A.bd_lof[e] = float(lo); A.bd_hif[e] = float(hi);
+        D.eta_hi[e] = D.eta_lo[e] = __int_as_float(-1);    // NaN: no warm start yet
+        P.lam[e] = 0.0;
+    }
+    if (e < (int64_t)A.M * A.K) {
+        P.kappa[e] = 0.0;
+        if (A.flo) {
+            const double lo = A.flo[e], hi = A.fhi[e];
+            A.bd_flo[e] = lo; A.bd_fhi[e] = hi;
+            A.bd_flof[e] = float(lo); A.bd_fhif[e] = float(hi);
+            D.s[e] = D.ys[e] = 0.f;                        // s = 0 clipped on the first update
+            D.sflag[e] = 0;
+        }
+    }
+    if (e < (int64_t)A.M * KMAX) D.Qhi[e] = D.Qlo[e] = __float2bfloat16_rn(0.f);
+    if (e < (int64_t)A.M * PRISM_NDIAG) P.diag[e] = 0.0;
+    if (e < A.M) {
+        const double tau = A.tau ? A.tau[e] : INFINITY;
+        if (isnan(tau) || tau < 0) atomicOr(A.err, ERR_CAP);
+        if (isfinite(tau)) A.err[2] = 1;
+        A.bd_tau[e] = tau;
+        A.bd_tauf[e] = float(tau);
+        D.rho_idx[e] = A.rho_idx;
+        D.active[e] = 1;
+        D.iters[e] = D.status[e] = 0;
+        D.nu[e] = D.theta[e] = 0.f;
+        D.dnu[e] = __int_as_float(0x7f7f7f7f);             // 3.4e38: no margin yet
+        P.skip[e] = P.done[e] = 0;
+        P.nu[e] = P.theta[e] = 0.0;
+        if (A.flo) D.rps[e] = D.rds[e] = 0.f;
+    }
+    if (e == 0) {
+        D.n_active[0] = D.n_active[1] = 0;
+        if (D.pcount) D.pcount[0] = D.pcount[1] = 0;
+        for (int q = 0; q < A.n_ctr; ++q) D.xq_ctr[q] = 0;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(*D.t0));
+    }
+}
+
+// The number of accounts that the polish left for another pass of the iterations.
+__global__ void k_unsettled(int M, const int* skip, const int* done, const int* status, int* n) {
+    int c = 0;
+    for (int a = threadIdx.x; a < M; a += blockDim.x)
+        c += !(skip[a] || done[a] == 1 || status[a] == PRISM_NUMERICAL_FAILURE);
+    c = __syncthreads_count(c > 0);                        // (threads with any: zero exactly when there is none)
+    if (threadIdx.x == 0) *n = c;
 }
 
 struct UnpackArgs {
@@ -199,12 +268,17 @@ __global__ void k_unpack(UnpackArgs A) {
 __global__ void k_capacity(int S, int N, int Npad, const int* sec_start, const double* LO, const double* UP,
                            const double* W0, const float* LOf, const float* UPf, const float* W0f,
                            const double* band_lo, const double* band_hi, const double* tau, int* status, int* skip,
-                           int* active) {
+                           int* active, double* W) {
     const int a = blockIdx.x;
     __shared__ double s_up[SMAX], s_lo[SMAX], s_kept[SMAX], s_forced[SMAX], s_w0[SMAX];
     __shared__ float f_up[SMAX], f_lo[SMAX];
     __shared__ int sec[SMAX + 1];
-    __shared__ int decided;
+    __shared__ int decided, rejected;             // rejected: nothing later writes the account's weights
+    auto no_weights = [&]() {
+        if (rejected)
+            for (int p = threadIdx.x; p < Npad; p += blockDim.x) W[(size_t)a * Npad + p] = 0.0;
+    };
+    if (threadIdx.x == 0) rejected = 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const size_t base = (size_t)a * Npad;
     for (int s = threadIdx.x; s <= S; s += blockDim.x) sec[s] = sec_start[s];
@@ -260,10 +334,11 @@ __global__ void k_capacity(int S, int N, int Npad, const int* sec_start, const d
                 status[a] = PRISM_NO_FEASIBLE_RETURN;
                 skip[a] = 1;
                 active[a] = 0;
+                rejected = 1;
             }
         }
         __syncthreads();
-        if (decided) return;
+        if (decided) { no_weights(); return; }
     }
     for (int s = warp; s < S; s += nw) {
         double su = 0, sl = 0, sk = 0, sf = 0, sw = 0;
@@ -294,8 +369,11 @@ __global__ void k_capacity(int S, int N, int Npad, const int* sec_start, const d
             status[a] = PRISM_NO_FEASIBLE_RETURN;
             skip[a] = 1;
             active[a] = 0;
+            rejected = 1;
         }
     }
+    __syncthreads();
+    no_weights();
 }
 
 // ---------------------------------------------------------------------------
@@ -638,11 +716,12 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     BlkArgs<double> P64;               // PLAIN_FP64: the FP64 per-account kernel's arguments
     BlkArgs<float> PK;                 // ragged books, packed layout: the FP32 per-account kernel's
     unsigned long long* t0_dev = nullptr;   // device clock at the start of the solve
+    char* inbox = nullptr;             // small host inputs (see stage_in)
     auto layout = [&](Arena& A, Dev& D, PolDev& P, BatchDev& BD, void** stage, int** member, int** err,
                       int** pwidx_dev, double** ragged_out) {
         BD.w0 = A.take<double>(MN); BD.lo = A.take<double>(MN); BD.up = A.take<double>(MN); BD.c = A.take<double>(MN);
         BD.w0f = A.take<float>(MN); BD.lof = A.take<float>(MN); BD.upf = A.take<float>(MN); BD.cf = A.take<float>(MN);
-        *member = A.take<int>(MN);
+        *member = A.take<int>(b->asset_idx ? MN : 0);
         *pwidx_dev = has_pw ? A.take<int>(MN) : nullptr;
         BD.band_lo = A.take<double>((size_t)M * S); BD.band_hi = A.take<double>((size_t)M * S);
         BD.band_lof = A.take<float>((size_t)M * S); BD.band_hif = A.take<float>((size_t)M * S);
@@ -721,6 +800,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         PK.plist = A.take<int>(lists ? (size_t)nnz : 0); PK.psec = A.take<int>(lists ? (size_t)M * (S + 1) : 0);
         PK.order = A.take<int>(lists ? M : 0); PK.queue = A.take<int>(4);
         t0_dev = A.take<unsigned long long>(1);
+        inbox = A.take<char>(SolveCache::BOX);
         PK.z = A.take<float>(np); PK.y = A.take<float>(np); PK.X = A.take<float>(np);
         PK.w0p = A.take<float>(np); PK.lop = A.take<float>(np); PK.upp = A.take<float>(np); PK.cp = A.take<float>(np);
         PK.pwp = A.take<int>(np);
@@ -753,6 +833,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         }
         if (!SC.pinned) {
             if (cudaMallocHost(&SC.pinned, 64) != cudaSuccess) { set_error("pinned alloc failed"); return PRISM_ERR_ALLOCATION; }
+            if (cudaMallocHost(&SC.box, 2 * SolveCache::BOX) != cudaSuccess) { cudaGetLastError(); SC.box = nullptr; }
             for (auto& e : SC.ev) cudaEventCreate(&e);
             if (cudaStreamCreateWithFlags(&SC.pst, cudaStreamNonBlocking) != cudaSuccess ||
                 cudaEventCreateWithFlags(&SC.ev_pol, cudaEventDisableTiming) != cudaSuccess) {
@@ -787,10 +868,25 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     SC.prof.on = o->profile != 0;
     cudaEventRecord(SC.ev[0], st);
     // ---- stage inputs on the device
+    // (small host arrays are gathered in pinned memory and go over in one copy per flush: each copy of
+    // its own from pageable memory takes 5 us and more of the host's time)
+    size_t box_used = 0, box_sent = 0;
     auto stage_in = [&](const void* src, void* dst, size_t bytes) -> const void* {
         if (is_dev(src)) return src;
+        const size_t room = (bytes + 255) / 256 * 256;
+        if (SC.box && room <= SolveCache::BOX / 4 && box_used + room <= SolveCache::BOX) {
+            std::memcpy(SC.box + box_used, src, bytes);
+            void* at = inbox + box_used;
+            box_used += room;
+            return at;
+        }
         cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
         return dst;
+    };
+    auto flush = [&]() {
+        if (box_used > box_sent)
+            cudaMemcpyAsync(inbox + box_sent, SC.box + box_sent, box_used - box_sent, cudaMemcpyHostToDevice, st);
+        box_sent = box_used;
     };
     PackArgs PA;
     PA.M = M; PA.N = N; PA.Npad = Npad; PA.nnz = nnz;
@@ -798,8 +894,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     PA.lo = (const double*)stage_in(b->lower, stage[1], nnz * 8);
     PA.up = (const double*)stage_in(b->upper, stage[2], nnz * 8);
     PA.tc = (const double*)stage_in(b->tc, stage[3], nnz * 8);
-    cudaMemcpyAsync(stage[4], offs.data(), (M + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, st);
-    PA.offsets = (const int64_t*)stage[4];
+    PA.offsets = (const int64_t*)stage_in(offs.data(), stage[4], (M + 1) * sizeof(int64_t));
     PA.asset_idx = b->asset_idx ? (const int32_t*)stage_in(b->asset_idx, stage[5], nnz * 4) : nullptr;
     PA.inv_perm = U.d_inv_perm;
     PA.W0 = BD.w0; PA.LO = BD.lo; PA.UP = BD.up; PA.C = BD.c;
@@ -821,45 +916,33 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         };
         pad(BD.w0, 8); pad(BD.lo, 8); pad(BD.up, 8); pad(BD.c, 8);
         pad(BD.w0f, 4); pad(BD.lof, 4); pad(BD.upf, 4); pad(BD.cf, 4);
-        pad(member, 4);
     }
     cudaMemsetAsync(err, 0, 16, st);
+    flush();
     if (nnz > 0) SC.prof.run(PRISM_K_PACK, 1, st, [&] { k_pack<<<(unsigned)cdiv64(nnz, 256), 256, 0, st>>>(PA); });
-    // bands and caps
+    // bands, caps, factor bounds and the accounts' state
     {
-        std::vector<double> blo, bhi, tau;
-        if ((rc = to_host(b->band_lo, (size_t)M * S, blo)) || (rc = to_host(b->band_hi, (size_t)M * S, bhi))) return rc;
-        if (b->turnover_cap) { if ((rc = to_host(b->turnover_cap, (size_t)M, tau))) return rc; }
-        else tau.assign(M, INFINITY);
-        for (size_t q = 0; q < blo.size(); ++q) {
-            if (std::isnan(blo[q]) || std::isnan(bhi[q]) || blo[q] > bhi[q]) {
-                set_error("band_lo <= band_hi required (no NaN)");
-                return PRISM_ERR_ARGUMENT;
-            }
-        }
-        bool cap_any = false;
-        for (int a = 0; a < M; ++a) {
-            if (std::isnan(tau[a]) || tau[a] < 0) { set_error("turnover_cap must be >= 0 or +inf"); return PRISM_ERR_ARGUMENT; }
-            cap_any |= std::isfinite(tau[a]);
-        }
-        std::vector<float> blof(blo.begin(), blo.end()), bhif(bhi.begin(), bhi.end()), tauf(tau.begin(), tau.end());
-        // the host vectors die at scope end: copy synchronously
-        PRISM_CUDA_TRY(cudaMemcpyAsync(BD.band_lo, blo.data(), blo.size() * 8, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaMemcpyAsync(BD.band_hi, bhi.data(), bhi.size() * 8, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaMemcpyAsync(BD.band_lof, blof.data(), blof.size() * 4, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaMemcpyAsync(BD.band_hif, bhif.data(), bhif.size() * 4, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaMemcpyAsync(BD.tau, tau.data(), M * 8, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaMemcpyAsync(BD.tauf, tauf.data(), M * 4, cudaMemcpyHostToDevice, st));
-        BD.has_cap = cap_any;
-        std::vector<float> lf(flo_h.begin(), flo_h.end()), hf(fhi_h.begin(), fhi_h.end());
+        SetupArgs SA = {};
+        SA.M = M; SA.S = S; SA.K = K;
+        int j0 = (int)std::lround(RHO_PER_DECADE * std::log10(std::max(o->rho0, 1e-12) / RHO_MIN));
+        SA.rho_idx = std::max(0, std::min(NRHO - 1, j0));
+        SA.n_ctr = 2 * SolveCache::MAXCH;
+        SA.band_lo = (const double*)stage_in(b->band_lo, BD.band_lo, (size_t)M * S * 8);
+        SA.band_hi = (const double*)stage_in(b->band_hi, BD.band_hi, (size_t)M * S * 8);
+        SA.tau = b->turnover_cap ? (const double*)stage_in(b->turnover_cap, BD.tau, (size_t)M * 8) : nullptr;
+        SA.bd_lo = BD.band_lo; SA.bd_hi = BD.band_hi; SA.bd_tau = BD.tau;
+        SA.bd_lof = BD.band_lof; SA.bd_hif = BD.band_hif; SA.bd_tauf = BD.tauf;
         if (has_fac_in) {
-            PRISM_CUDA_TRY(cudaMemcpyAsync(BD.flo, flo_h.data(), flo_h.size() * 8, cudaMemcpyHostToDevice, st));
-            PRISM_CUDA_TRY(cudaMemcpyAsync(BD.fhi, fhi_h.data(), fhi_h.size() * 8, cudaMemcpyHostToDevice, st));
-            PRISM_CUDA_TRY(cudaMemcpyAsync(BD.flof, lf.data(), lf.size() * 4, cudaMemcpyHostToDevice, st));
-            PRISM_CUDA_TRY(cudaMemcpyAsync(BD.fhif, hf.data(), hf.size() * 4, cudaMemcpyHostToDevice, st));
+            SA.flo = (const double*)stage_in(flo_h.data(), BD.flo, flo_h.size() * 8);
+            SA.fhi = (const double*)stage_in(fhi_h.data(), BD.fhi, fhi_h.size() * 8);
+            SA.bd_flo = BD.flo; SA.bd_fhi = BD.fhi; SA.bd_flof = BD.flof; SA.bd_fhif = BD.fhif;
             BD.has_fac = true;
         }
-        PRISM_CUDA_TRY(cudaStreamSynchronize(st));
+        SA.D = D; SA.P = P; SA.err = err;
+        SA.D.t0 = t0_dev;
+        const int64_t n = (int64_t)M * std::max(std::max(S, K), KMAX);
+        flush();
+        SC.prof.run(PRISM_K_OTHER, 1, st, [&] { k_setup<<<(unsigned)cdiv64(n, 256), 256, 0, st>>>(SA); });
     }
     // lots and tilts
     if (has_lots || has_tilt) {
@@ -884,16 +967,18 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         CA.pw_idx = pwidx; CA.bp = BD.pw_bp; CA.sl = BD.pw_sl; CA.phi_lo = (double*)stage[6];
         CA.bpf = BD.pw_bpf; CA.slf = BD.pw_slf; CA.nbp = BD.pw_nbp; CA.err = err;
         if (pwidx) cudaMemsetAsync(pwidx, 0xff, MN * 4, st);
+        flush();
         SC.prof.run(PRISM_K_PACK, b->w_bench ? 2 : 1, st, [&] {
             if (b->w_bench) k_bench_factors<<<M, 256, 0, st>>>(CA);
             if (nnz > 0) k_costs<<<(unsigned)cdiv64(nnz, 128), 128, 0, st>>>(CA);
         });
     }
     {
-        int flags[2] = {0, 0};
-        PRISM_CUDA_TRY(cudaMemcpyAsync(flags, err, 8, cudaMemcpyDeviceToHost, st));
+        int* flags = SC.pinned + 4;
+        PRISM_CUDA_TRY(cudaMemcpyAsync(flags, err, 12, cudaMemcpyDeviceToHost, st));
         PRISM_CUDA_TRY(cudaStreamSynchronize(st));
         const int herr = flags[0];
+        BD.has_cap = flags[2] != 0;
         if (!has_lots && !flags[1]) pwidx = nullptr;      // every tilt is zero: plain costs throughout
         struct { int bit, code; const char* text; } lot_errors[] = {
             {ERR_LOT_OFFSETS, PRISM_ERR_ARGUMENT, "lot_offsets must be nondecreasing"},
@@ -902,7 +987,9 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
             {ERR_LOT_DATA, PRISM_ERR_ARGUMENT, "bad lot data"},
             {ERR_LOT_SUM, PRISM_ERR_ARGUMENT, "lot sizes of an entry must sum to its w0"},
             {ERR_BENCH, PRISM_ERR_ARGUMENT, "w_bench must be finite"},
-            {ERR_TILT, PRISM_ERR_ARGUMENT, "mu_tilt must be finite"}};
+            {ERR_TILT, PRISM_ERR_ARGUMENT, "mu_tilt must be finite"},
+            {ERR_BAND, PRISM_ERR_ARGUMENT, "band_lo <= band_hi required (no NaN)"},
+            {ERR_CAP, PRISM_ERR_ARGUMENT, "turnover_cap must be >= 0 or +inf"}};
         for (auto& q : lot_errors)
             if (herr & q.bit) { set_error(q.text); return q.code; }
         if (herr) {
@@ -1014,52 +1101,15 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     }
     if (acct && b->asset_idx)
         PRISM_CUDA_TRY(cudaMemcpyAsync(PK.order, order_h.data(), (size_t)M * 4, cudaMemcpyHostToDevice, st));
-    // ---- control init
-    {
-        int j0 = (int)std::lround(RHO_PER_DECADE * std::log10(std::max(o->rho0, 1e-12) / RHO_MIN));
-        j0 = std::max(0, std::min(NRHO - 1, j0));
-        std::vector<int> h(M, j0);
-        PRISM_CUDA_TRY(cudaMemcpyAsync(D.rho_idx, h.data(), M * 4, cudaMemcpyHostToDevice, st));
-        std::vector<int> one(M, 1);
-        PRISM_CUDA_TRY(cudaMemcpyAsync(D.active, one.data(), M * 4, cudaMemcpyHostToDevice, st));
-        PRISM_CUDA_TRY(cudaStreamSynchronize(st));
-        cudaMemsetAsync(D.iters, 0, M * 4, st);
-        cudaMemsetAsync(D.status, 0, M * 4, st);
-        cudaMemsetAsync(D.nu, 0, M * 4, st);
-        cudaMemsetAsync(D.dnu, 0x7f, M * 4, st);                    // 3.4e38: no margin yet
-        cudaMemsetAsync(D.theta, 0, M * 4, st);
-        cudaMemsetAsync(D.eta_hi, 0xff, (size_t)M * S * 4, st);   // NaN: no warm start yet
-        cudaMemsetAsync(D.eta_lo, 0xff, (size_t)M * S * 4, st);
-        cudaMemsetAsync(P.skip, 0, M * 4, st);
-        cudaMemsetAsync(P.done, 0, M * 4, st);
-        cudaMemsetAsync(P.diag, 0, (size_t)M * PRISM_NDIAG * 8, st);
-        cudaMemsetAsync(P.W, 0, MN * 8, st);
-        cudaMemsetAsync(P.nu, 0, M * 8, st);
-        cudaMemsetAsync(P.theta, 0, M * 8, st);
-        cudaMemsetAsync(P.lam, 0, (size_t)M * S * 8, st);
-        cudaMemsetAsync(P.kappa, 0, (size_t)M * K * 8, st);
-        if (BD.has_fac) {
-            cudaMemsetAsync(D.s, 0, (size_t)M * K * 4, st);     // s = 0 clipped on the first update
-            cudaMemsetAsync(D.ys, 0, (size_t)M * K * 4, st);
-            cudaMemsetAsync(D.sflag, 0, (size_t)M * K * 4, st);
-            cudaMemsetAsync(D.rps, 0, M * 4, st);
-            cudaMemsetAsync(D.rds, 0, M * 4, st);
-        }
-        cudaMemsetAsync(D.X, 0, MN * 4, st);
-        cudaMemsetAsync(D.Xhi, 0, MN * 2, st);
-        cudaMemsetAsync(D.Xlo, 0, MN * 2, st);
+    // ---- control init (see k_setup)
+    if (!acct) {
         cudaMemsetAsync(D.v, 0, MN * 4, st);
-        cudaMemsetAsync(D.Qhi, 0, (size_t)M * KMAX * 2, st);
-        cudaMemsetAsync(D.Qlo, 0, (size_t)M * KMAX * 2, st);
-        cudaMemsetAsync(D.n_active, 0, 8, st);
         if (D.stats) cudaMemsetAsync(D.stats, 0, 32, st);
-        if (D.pcount) cudaMemsetAsync(D.pcount, 0, 16, st);
-        if (D.xq_ctr) cudaMemsetAsync(D.xq_ctr, 0, 2 * SolveCache::MAXCH * sizeof(unsigned), st);
     }
-    SC.prof.run(PRISM_K_OTHER, 2, st, [&] {
+    SC.prof.run(PRISM_K_OTHER, acct ? 1 : 2, st, [&] {
         k_capacity<<<M, 256, 0, st>>>(S, N, Npad, U.d_sec_start, BD.lo, BD.up, BD.w0, BD.lof, BD.upf, BD.w0f,
-                                      BD.band_lo, BD.band_hi, BD.tau, D.status, P.skip, D.active);
-        launch_init_state(D, st);
+                                      BD.band_lo, BD.band_hi, BD.tau, D.status, P.skip, D.active, P.W);
+        if (!acct) launch_init_state(D, st);
     });
     if (D.fused) {
         SC.prof.run(PRISM_K_OTHER, 1, st, [&] { launch_uniform(D, (float*)D.lo_u, (float*)D.c_u, st); });
@@ -1364,6 +1414,10 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         if (polish_rounds(false) < 0) { set_error("polish failed"); return PRISM_ERR_CUDA; }
     }
     for (int retry = 0; retry < 2; ++retry) {
+        SC.prof.run(PRISM_K_OTHER, 1, st, [&] { k_unsettled<<<1, 1024, 0, st>>>(M, P.skip, P.done, D.status, err + 3); });
+        PRISM_CUDA_TRY(cudaMemcpyAsync(SC.pinned + 8, err + 3, 4, cudaMemcpyDeviceToHost, st));
+        PRISM_CUDA_TRY(cudaStreamSynchronize(st));
+        if (SC.pinned[8] == 0) break;
         std::vector<int> done(M), skip(M), status(M);
         cudaMemcpyAsync(done.data(), P.done, M * 4, cudaMemcpyDeviceToHost, st);
         cudaMemcpyAsync(skip.data(), P.skip, M * 4, cudaMemcpyDeviceToHost, st);
@@ -1433,10 +1487,23 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     const bool w_dev = is_dev(res->w);
     UA.out = w_dev ? res->w : ragged_out;
     if (nnz > 0) SC.prof.run(PRISM_K_UNPACK, 1, st, [&] { k_unpack<<<(unsigned)cdiv64(nnz, 256), 256, 0, st>>>(UA); });
-    if (!w_dev) cudaMemcpyAsync(res->w, ragged_out, nnz * 8, cudaMemcpyDeviceToHost, st);
+    // (small outputs to host memory come back through the box, and are handed out once all are there)
+    struct Out { void* dst; const char* at; size_t bytes; } outs[8];
+    int n_out = 0;
+    size_t out_used = 0;
     auto out = [&](void* dst, const void* src, size_t bytes) {
-        if (dst) cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, st);
+        if (!dst) return;
+        const size_t room = (bytes + 255) / 256 * 256;
+        if (SC.box && bytes && room <= SolveCache::BOX / 4 && out_used + room <= SolveCache::BOX && !is_dev(dst)) {
+            char* at = SC.box + SolveCache::BOX + out_used;
+            out_used += room;
+            cudaMemcpyAsync(at, src, bytes, cudaMemcpyDeviceToHost, st);
+            outs[n_out++] = {dst, at, bytes};
+            return;
+        }
+        cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, st);
     };
+    if (!w_dev) out(res->w, ragged_out, nnz * 8);
     out(res->status, D.status, M * 4);
     out(res->iters, D.iters, M * 4);
     out(res->nu, P.nu, M * 8);
@@ -1447,6 +1514,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     cudaEventRecord(SC.ev[5], st);
     cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) { set_error(std::string("solve failed: ") + cudaGetErrorString(e)); return PRISM_ERR_CUDA; }
+    for (int q = 0; q < n_out; ++q) std::memcpy(outs[q].dst, outs[q].at, outs[q].bytes);
     e = cudaGetLastError();
     if (e != cudaSuccess) { set_error(std::string("solve failed: ") + cudaGetErrorString(e)); return PRISM_ERR_CUDA; }
     res->t_phase_ms[0] = ms_between(SC.ev[0], SC.ev[1]);
