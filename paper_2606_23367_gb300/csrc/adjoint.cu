@@ -26,6 +26,8 @@
 // (a dependent working row gets kappa = 0). Sums over accounts run in a fixed order.
 #include <algorithm>
 #include <cstring>
+#include <utility>
+#include <vector>
 
 #include "common.cuh"
 #include "polish.h"
@@ -36,6 +38,7 @@ namespace {
 
 constexpr int AB = 256;                // threads per adjoint block (one block per account)
 constexpr int AMAXROWS = PMAXROWS;     // working rows
+constexpr int ADINV = 256;             // free weights whose 1 / d lives in shared memory
 constexpr int AYS = AMAXROWS + 1;      // row stride of Y: column 0 = g_F, columns 1..m = E_F'
 
 struct AdjArgs {
@@ -56,6 +59,8 @@ struct AdjShared {
     double C[KMAX][KMAX + 1];
     double T[KMAX][AYS];
     double Ldinv[KMAX];
+    double dinv[ADINV];                 // 1 / d of the first free weights: a division costs about 30 FP64
+                                        // multiply-adds, at two a cycle and SM
     double Sm[AMAXROWS][AMAXROWS + 1];
     double r[AMAXROWS], kappa[AMAXROWS];
     double ft[KMAX], fh[KMAX];
@@ -141,10 +146,13 @@ __global__ void __launch_bounds__(AB) k_adjoint(AdjArgs A) {
     for (int q = tid; q < nF; q += AB) {
         const int p = Fl[q];
         const double di = 1.0 / A.d64[p];
+        if (q < ADINV) sh.dinv[q] = di;
         double* Yq = Y + (size_t)q * AYS;
         Yq[0] = A.G[base + p] * di;
         for (int r = 0; r < m; ++r) Yq[1 + r] = row_coef(A, sh, r, p, FL[p]) * di;
     }
+    __syncthreads();
+    auto inv_d = [&](int q, int p) { return q < ADINV ? sh.dinv[q] : 1.0 / A.d64[p]; };
     // ---- C = F^{-1} + B_F' D_F^{-1} B_F and its Cholesky factor (L D L', then L)
     for (int e2 = tid; e2 < K * K; e2 += AB) {
         const int r = e2 / K, c = e2 % K;
@@ -152,7 +160,7 @@ __global__ void __launch_bounds__(AB) k_adjoint(AdjArgs A) {
         double acc = (r == c) ? 1.0 / A.f64[r] : 0.0;
         for (int q = 0; q < nF; ++q) {
             const int p = Fl[q];
-            acc += A.B64[(size_t)p * K + r] * A.B64[(size_t)p * K + c] / A.d64[p];
+            acc += A.B64[(size_t)p * K + r] * A.B64[(size_t)p * K + c] * inv_d(q, p);
         }
         sh.C[r][c] = acc;
     }
@@ -172,14 +180,13 @@ __global__ void __launch_bounds__(AB) k_adjoint(AdjArgs A) {
         if (tid == 0) atomicOr(A.err, 2);
         return;
     }
-    for (int c = tid; c < K; c += AB) sh.Ldinv[c] = sqrt(sh.C[c][c]);
+    for (int c = tid; c < K; c += AB) sh.Ldinv[c] = 1.0 / sqrt(sh.C[c][c]);
     __syncthreads();
     for (int e2 = tid; e2 < K * K; e2 += AB) {
         const int r = e2 / K, c = e2 % K;
-        if (c < r) sh.C[r][c] /= sh.Ldinv[c];
+        if (c < r) sh.C[r][c] *= sh.Ldinv[c];
     }
     __syncthreads();
-    for (int c = tid; c < K; c += AB) { sh.C[c][c] = sh.Ldinv[c]; sh.Ldinv[c] = 1.0 / sh.Ldinv[c]; }
     // ---- Woodbury: Y <- Y - D^{-1} B_F C^{-1} B_F' Y
     for (int e2 = tid; e2 < K * nc1; e2 += AB) {
         const int k = e2 / nc1, c = e2 % nc1;
@@ -211,7 +218,7 @@ __global__ void __launch_bounds__(AB) k_adjoint(AdjArgs A) {
         const int p = Fl[q];
         double acc = 0.0;
         for (int k = 0; k < K; ++k) acc += A.B64[(size_t)p * K + k] * sh.T[k][c];
-        Y[(size_t)q * AYS + c] -= acc / A.d64[p];
+        Y[(size_t)q * AYS + c] -= acc * inv_d(q, p);
     }
     __syncthreads();
     // ---- Schur complement S = E Y_E, r = E Y_g; pivoted elimination, kappa = S^+ r
@@ -265,14 +272,24 @@ __global__ void __launch_bounds__(AB) k_adjoint(AdjArgs A) {
     }
     __syncthreads();
     // ---- F t = f o (B_F' u) and F h = f o (B' w)
-    for (int k = tid; k < K; k += AB) {
+    static_assert(AB / KMAX == 4, "four lanes per factor");
+    {
+        const int k = tid >> 2, sub = tid & 3;
         double t = 0.0, h = 0.0;
-        for (int q = 0; q < nF; ++q) t += A.B64[(size_t)Fl[q] * K + k] * Y[(size_t)q * AYS];
-        for (int q = 0; q < nNZ; ++q) h += A.B64[(size_t)NZ[q] * K + k] * W[NZ[q]];
-        sh.ft[k] = A.f64[k] * t;
-        sh.fh[k] = A.f64[k] * h;
-        A.Ft[(size_t)a * K + k] = sh.ft[k];
-        A.Fh[(size_t)a * K + k] = sh.fh[k];
+        if (k < K) {
+#pragma unroll 4
+            for (int q = sub; q < nF; q += 4) t += A.B64[(size_t)Fl[q] * K + k] * Y[(size_t)q * AYS];
+#pragma unroll 4
+            for (int q = sub; q < nNZ; q += 4) h += A.B64[(size_t)NZ[q] * K + k] * W[NZ[q]];
+        }
+        t += __shfl_xor_sync(0xffffffffu, t, 2); h += __shfl_xor_sync(0xffffffffu, h, 2);
+        t += __shfl_xor_sync(0xffffffffu, t, 1); h += __shfl_xor_sync(0xffffffffu, h, 1);
+        if (k < K && sub == 0) {
+            sh.ft[k] = A.f64[k] * t;
+            sh.fh[k] = A.f64[k] * h;
+            A.Ft[(size_t)a * K + k] = sh.ft[k];
+            A.Fh[(size_t)a * K + k] = sh.fh[k];
+        }
     }
     __syncthreads();
     // ---- dL/dw0 of every entry of the account
@@ -343,6 +360,25 @@ __global__ void k_adjoint_gather(int M, int Npad, int64_t nnz, const int64_t* of
     out[e] = DW0[ragged_slot(offsets, asset_idx, inv_perm, M, Npad, e)];
 }
 
+// Arrays that share one allocation: a cudaMalloc and its cudaFree take 20 us and more each, and a training
+// step made and freed 21 of them for every backward state.
+struct Block {
+    std::vector<std::pair<void**, size_t>> at;
+    size_t bytes = 0;
+    template <class T>
+    void place(T** p, size_t n) {
+        at.push_back({(void**)p, bytes});
+        bytes += (std::max<size_t>(n, 1) * sizeof(T) + 255) / 256 * 256;
+    }
+    bool allocate(std::vector<void*>& owner) {
+        char* base = nullptr;
+        if (cudaMalloc((void**)&base, bytes) != cudaSuccess) { cudaGetLastError(); return false; }
+        owner.push_back(base);
+        for (auto& q : at) *q.first = base + q.second;
+        return true;
+    }
+};
+
 template <class T>
 bool dev_ptr(const T* p) {
     cudaPointerAttributes at;
@@ -360,21 +396,15 @@ int make_backward_state(const prism_universe* uh, const PolDev& P, const int* st
     auto* s = new prism_state();
     s->uh = uh; s->device = U.device; s->M = P.M; s->N = P.N; s->Npad = P.Npad; s->K = P.K; s->S = P.S; s->nnz = nnz;
     const size_t MN = (size_t)P.M * P.Npad;
-    auto take = [&](size_t bytes) -> void* {
-        void* q = nullptr;
-        if (cudaMalloc(&q, std::max<size_t>(bytes, 16)) != cudaSuccess) return nullptr;
-        s->blocks.push_back(q);
-        return q;
-    };
-    s->offsets = (int64_t*)take((P.M + 1) * 8);
-    s->asset_idx = asset_idx_dev ? (int32_t*)take(nnz * 4) : nullptr;
-    s->W = (double*)take(MN * 8);
-    s->flags = (uint8_t*)take(MN);
-    s->wband = (int*)take((size_t)P.M * P.S * 4);
-    s->wcap = (int*)take(P.M * 4);
-    s->status = (int*)take(P.M * 4);
-    for (void* q : s->blocks)
-        if (!q) { prism_free_state(s); set_error("cudaMalloc (backward state) failed"); return PRISM_ERR_ALLOCATION; }
+    Block blk;
+    blk.place(&s->offsets, P.M + 1);
+    if (asset_idx_dev) blk.place(&s->asset_idx, nnz);
+    blk.place(&s->W, MN);
+    blk.place(&s->flags, MN);
+    blk.place(&s->wband, (size_t)P.M * P.S);
+    blk.place(&s->wcap, P.M);
+    blk.place(&s->status, P.M);
+    if (!blk.allocate(s->blocks)) { prism_free_state(s); set_error("cudaMalloc (backward state) failed"); return PRISM_ERR_ALLOCATION; }
     cudaMemcpyAsync(s->offsets, offsets_dev, (P.M + 1) * 8, cudaMemcpyDeviceToDevice, st);
     if (asset_idx_dev) cudaMemcpyAsync(s->asset_idx, asset_idx_dev, nnz * 4, cudaMemcpyDeviceToDevice, st);
     cudaMemcpyAsync(s->W, P.W, MN * 8, cudaMemcpyDeviceToDevice, st);
@@ -398,28 +428,24 @@ extern "C" int prism_solve_batch_backward(prism_state* s, const double* dL_dw, d
     const size_t MN = (size_t)M * Npad;
     if (!s->G) {
         s->fmax = std::min(Npad, 2048);
-        auto take = [&](size_t bytes) -> void* {
-            void* q = nullptr;
-            if (cudaMalloc(&q, std::max<size_t>(bytes, 16)) != cudaSuccess) return nullptr;
-            s->blocks.push_back(q);
-            return q;
-        };
-        s->G = (double*)take(MN * 8);
-        s->U = (double*)take(MN * 8);
-        s->DW0 = (double*)take(MN * 8);
-        s->Fh = (double*)take((size_t)M * K * 8);
-        s->Ft = (double*)take((size_t)M * K * 8);
-        s->Y = (double*)take((size_t)M * s->fmax * AYS * 8);
-        s->Flist = (int*)take((size_t)M * s->fmax * 4);
-        s->NZlist = (int*)take(MN * 4);
-        s->err = (int*)take(16);
-        s->out_dmu = (double*)take((size_t)N * 8);
-        s->out_dd = (double*)take((size_t)N * 8);
-        s->out_dB = (double*)take((size_t)N * K * 8);
-        s->out_dw0 = (double*)take(std::max<int64_t>(s->nnz, 1) * 8);
-        s->in_g = (double*)take(std::max<int64_t>(s->nnz, 1) * 8);
-        for (void* q : s->blocks)
-            if (!q) { set_error("cudaMalloc (backward scratch) failed"); return PRISM_ERR_ALLOCATION; }
+        // (what has to be zero at the start of a call first, so that one memset clears it)
+        Block blk;
+        blk.place(&s->G, MN);
+        blk.place(&s->U, MN);
+        blk.place(&s->DW0, MN);
+        blk.place(&s->Fh, (size_t)M * K);
+        blk.place(&s->Ft, (size_t)M * K);
+        blk.place(&s->err, 4);
+        s->zeroed = blk.bytes;
+        blk.place(&s->Y, (size_t)M * s->fmax * AYS);
+        blk.place(&s->Flist, (size_t)M * s->fmax);
+        blk.place(&s->NZlist, MN);
+        blk.place(&s->out_dmu, N);
+        blk.place(&s->out_dd, N);
+        blk.place(&s->out_dB, (size_t)N * K);
+        blk.place(&s->out_dw0, std::max<int64_t>(s->nnz, 1));
+        blk.place(&s->in_g, std::max<int64_t>(s->nnz, 1));
+        if (!blk.allocate(s->blocks)) { s->G = nullptr; set_error("cudaMalloc (backward scratch) failed"); return PRISM_ERR_ALLOCATION; }
     }
     cudaStream_t st = 0;
     const double* g_dev = dL_dw;
@@ -427,12 +453,7 @@ extern "C" int prism_solve_batch_backward(prism_state* s, const double* dL_dw, d
         PRISM_CUDA_TRY(cudaMemcpy(s->in_g, dL_dw, s->nnz * 8, cudaMemcpyHostToDevice));
         g_dev = s->in_g;
     }
-    cudaMemsetAsync(s->G, 0, MN * 8, st);
-    cudaMemsetAsync(s->U, 0, MN * 8, st);
-    cudaMemsetAsync(s->DW0, 0, MN * 8, st);
-    cudaMemsetAsync(s->Fh, 0, (size_t)M * K * 8, st);
-    cudaMemsetAsync(s->Ft, 0, (size_t)M * K * 8, st);
-    cudaMemsetAsync(s->err, 0, 16, st);
+    cudaMemsetAsync(s->G, 0, s->zeroed, st);
     if (s->nnz > 0)
         k_adjoint_scatter<<<(unsigned)cdiv64(s->nnz, 256), 256, 0, st>>>(M, Npad, s->nnz, s->offsets, s->asset_idx,
                                                                           U.d_inv_perm, g_dev, s->G);

@@ -67,6 +67,7 @@ struct Universe {
     float* d_CinvF32 = nullptr;    // NRHO x K x K, ((2F + rho_j I)^{-1} + G_j)^{-1}, FP32 B
     float* d_CinvF16 = nullptr;    // the same for the BF16-rounded B
     double dmin = 0.0;             // smallest idiosyncratic variance d_i (strong convexity of the risk)
+    char* d_block = nullptr;       // the device memory that every array above lies in
     size_t bytes = 0;
     cudaStream_t stream = nullptr;
 };
@@ -125,6 +126,7 @@ struct prism_state {
     std::vector<void*> blocks;        // every device allocation above and the scratch below
     // backward scratch (allocated on first use)
     int fmax = 0;
+    size_t zeroed = 0;                // bytes from G on that a call starts with at zero
     double *G = nullptr, *U = nullptr, *DW0 = nullptr, *Fh = nullptr, *Ft = nullptr, *Y = nullptr;
     int *Flist = nullptr, *NZlist = nullptr, *err = nullptr;
     double *out_dmu = nullptr, *out_dd = nullptr, *out_dB = nullptr, *out_dw0 = nullptr, *in_g = nullptr;

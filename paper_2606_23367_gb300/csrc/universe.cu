@@ -25,10 +25,11 @@ const char* last_error() { return g_last_error.c_str(); }
 // G_j[k1][k2] = sum_i B[i][k1] B[i][k2] / (2 d_i + rho_j), FP32 products summed
 // in FP32 over chunks of 128 assets and in FP64 across chunks. One block per
 // (j, 8-row stripe of k1); B rows staged through shared memory.
-template <typename TB>
-__global__ void k_gram(const TB* __restrict__ B, const float* __restrict__ d, int N, int K,
-                       double* __restrict__ G) {
+// blockIdx.z: B in FP32 or as rounded to BF16.
+__global__ void k_gram(const float* __restrict__ B32, const __nv_bfloat16* __restrict__ B16,
+                       const float* __restrict__ d, int N, int K, double* __restrict__ Gs) {
     const int j = blockIdx.x;
+    double* G = Gs + (size_t)blockIdx.z * NRHO * K * K;
     const int k1_0 = blockIdx.y * 8;
     const float rho = float(RHO_MIN * pow(10.0, double(j) / RHO_PER_DECADE));
     __shared__ float sB[128][KMAX + 1];
@@ -43,7 +44,7 @@ __global__ void k_gram(const TB* __restrict__ B, const float* __restrict__ d, in
         for (int e = t; e < 128 * K; e += 256) {
             int r = e / K, c = e % K;
             int i = i0 + r;
-            sB[r][c] = (i < N) ? float(B[(size_t)i * K + c]) : 0.f;
+            sB[r][c] = (i < N) ? (blockIdx.z ? __bfloat162float(B16[(size_t)i * K + c]) : B32[(size_t)i * K + c]) : 0.f;
         }
         for (int r = t; r < 128; r += 256) {
             int i = i0 + r;
@@ -67,71 +68,94 @@ __global__ void k_gram(const TB* __restrict__ B, const float* __restrict__ d, in
     }
 }
 
-// Cinv_j = ((2F)^{-1} + G_j)^{-1} by an FP64 Cholesky factorisation in shared
-// memory, then an explicit inverse (columns by forward/back substitution). With
-// `split` the diagonal term is (2 f_k + rho_j)^{-1} instead: the capacitance of the
-// x-update when the factor exposures are split off with the same penalty. Gout, when
-// given, receives the FP32 copy of G_j.
-__global__ void k_cinv(const double* __restrict__ G, const double* __restrict__ f, int K,
-                       float* __restrict__ Cinv, int split, float* __restrict__ Gout) {
-    const int j = blockIdx.x;
-    __shared__ double L[KMAX][KMAX + 1];
-    const int t = threadIdx.x;   // 64 threads
+// Cinv_j = ((2F)^{-1} + G_j)^{-1} in FP64 (Gauss-Jordan, positive definite, so without pivoting; each step
+// from one buffer into the other, one barrier a step), rounded to FP32. blockIdx.y: bit 0 the BF16 B, bit
+// 1 the capacitance of the x-update when the factor exposures are split off with the same
+// penalty, whose diagonal term is (2 f_k + rho_j)^{-1}. A block per inverse, all 4 x 33 in one launch:
+// bound by the FP64 rate, K^3 / 2 cycles each. (Four launches of one 64-thread Cholesky per inverse, a
+// thread per column of it, took 0.6 of the 1.4 ms of a 2,000 x 32 universe.)
+struct CinvArgs {
+    const double* G;                       // 2 x NRHO x K x K
+    const double* f;
+    int K;
+    float* out[4];
+    float* G_out[2];                       // FP32 copies of the Gram matrices
+};
+
+__global__ void __launch_bounds__(256) k_cinv(CinvArgs A) {
+    extern __shared__ double cinv_smem[];
+    const int K = A.K, ld = K + 1, j = blockIdx.x, which = blockIdx.y, t = threadIdx.x;
+    const int lane = t & 31, warp = t >> 5, NW = blockDim.x >> 5;
+    double *from = cinv_smem, *to = cinv_smem + K * ld;
+    const double* G = A.G + ((size_t)(which & 1) * NRHO + j) * K * K;
     const double rho = RHO_MIN * pow(10.0, double(j) / RHO_PER_DECADE);
     for (int e = t; e < K * K; e += blockDim.x) {
-        int r = e / K, c = e % K;
-        double v = G[((size_t)j * K + r) * K + c];
-        if (Gout) Gout[((size_t)j * K + r) * K + c] = float(v);
-        if (r == c) v += split ? 1.0 / (2.0 * f[r] + rho) : 1.0 / (2.0 * f[r]);
-        L[r][c] = v;
+        const int r = e / K, c = e - r * K;
+        double v = G[e];
+        if (which < 2) A.G_out[which][(size_t)j * K * K + e] = float(v);
+        if (r == c) v += (which & 2) ? 1.0 / (2.0 * A.f[r] + rho) : 1.0 / (2.0 * A.f[r]);
+        from[r * ld + c] = v;
     }
     __syncthreads();
-    // right-looking Cholesky, lower triangle
-    for (int c = 0; c < K; ++c) {
-        if (t == 0) L[c][c] = sqrt(L[c][c]);
+    for (int k = 0; k < K; ++k) {
+        const double ip = 1.0 / from[k * ld + k];
+        for (int r = warp; r < K; r += NW) {
+            const double m = -from[r * ld + k] * ip;
+            for (int c = lane; c < K; c += 32) {
+                const double p = from[k * ld + c];
+                double q = (r == k) ? p * ip : fma(m, p, from[r * ld + c]);
+                if (c == k) q = (r == k) ? ip : m;
+                to[r * ld + c] = q;
+            }
+        }
         __syncthreads();
-        for (int r = c + 1 + t; r < K; r += blockDim.x) L[r][c] /= L[c][c];
-        __syncthreads();
-        for (int r = c + 1 + t; r < K; r += blockDim.x)
-            for (int q = c + 1; q <= r; ++q) L[r][q] -= L[r][c] * L[q][c];
-        __syncthreads();
+        double* x = from; from = to; to = x;
     }
-    // column t of the inverse: solve L L' x = e_t
-    if (t < K) {
-        double x[KMAX];
-        for (int r = 0; r < K; ++r) {
-            double s = (r == t) ? 1.0 : 0.0;
-            for (int q = 0; q < r; ++q) s -= L[r][q] * x[q];
-            x[r] = s / L[r][r];
-        }
-        for (int r = K - 1; r >= 0; --r) {
-            double s = x[r];
-            for (int q = r + 1; q < K; ++q) s -= L[q][r] * x[q];
-            x[r] = s / L[r][r];
-        }
-        for (int r = 0; r < K; ++r) Cinv[((size_t)j * K + r) * K + t] = float(x[r]);
+    float* out = A.out[which] + (size_t)j * K * K;
+    for (int e = t; e < K * K; e += blockDim.x) {
+        const int r = e / K, c = e - r * K;
+        out[e] = float(from[r * ld + c]);
     }
 }
 
-__global__ void k_convert_B(const double* __restrict__ B64, int Npad, int K, float* __restrict__ B32,
-                            float* __restrict__ B32p, __nv_bfloat16* __restrict__ B16, __nv_bfloat16* __restrict__ Bt16,
-                            __nv_bfloat16* __restrict__ B16p, __nv_bfloat16* __restrict__ Bt16p) {
-    size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (size_t)Npad * K) return;
-    int i = int(e / K), k = int(e % K);
-    double b = B64[e];
-    B32[e] = float(b);
-    B32p[(size_t)i * KMAX + k] = float(b);
-    __nv_bfloat16 h = __float2bfloat16_rn(float(b));
-    B16[e] = h;
-    Bt16[(size_t)k * Npad + i] = h;
-    B16p[(size_t)i * KMAX + k] = h;
-    Bt16p[(size_t)k * Npad + i] = h;
-}
+// The copies of B in sorted order from the caller's (a warp per position; padding rows are zero), and
+// sum_k |B_ik|. A non-finite entry sets *bad.
+struct ConvArgs {
+    const double* raw;                     // N x K, the caller's order
+    const int* perm;                       // sorted position -> asset
+    int N, Npad, K;
+    double* B64;
+    float *B32, *B32p;
+    __nv_bfloat16 *B16, *Bt16, *B16p, *Bt16p;
+    double* Bn1;
+    float* Bn1f;
+    int* bad;
+};
 
-__global__ void k_bf16_to_float(const __nv_bfloat16* __restrict__ a, float* __restrict__ b, size_t n) {
-    size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < n) b[e] = __bfloat162float(a[e]);
+__global__ void k_convert_B(ConvArgs A) {
+    const int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (p >= A.Npad) return;
+    const int K = A.K;
+    const double* row = p < A.N ? A.raw + (size_t)A.perm[p] * K : nullptr;
+    double n1 = 0.0;
+    for (int k = lane; k < KMAX; k += 32) {
+        const double b = (row && k < K) ? row[k] : 0.0;
+        const float f = float(b);
+        const __nv_bfloat16 h = __float2bfloat16_rn(f);
+        if (!isfinite(b)) *A.bad = 1;
+        n1 += fabs(b);
+        if (k < K) {
+            A.B64[(size_t)p * K + k] = b;
+            A.B32[(size_t)p * K + k] = f;
+            A.B16[(size_t)p * K + k] = h;
+            A.Bt16[(size_t)k * A.Npad + p] = h;
+        }
+        A.B32p[(size_t)p * KMAX + k] = f;
+        A.B16p[(size_t)p * KMAX + k] = h;
+        A.Bt16p[(size_t)k * A.Npad + p] = h;
+    }
+    n1 = warp_sum(n1);
+    if (lane == 0) { A.Bn1[p] = n1; A.Bn1f[p] = float(n1); }
 }
 
 static bool is_device_ptr(const void* p) {
@@ -141,6 +165,16 @@ static bool is_device_ptr(const void* p) {
         return false;
     }
     return attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged;
+}
+
+// Whether a kernel on device `dev` may read p where it is.
+static bool on_device(const void* p, int dev) {
+    cudaPointerAttributes attr;
+    if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return attr.type == cudaMemoryTypeManaged || (attr.type == cudaMemoryTypeDevice && attr.device == dev);
 }
 
 // Copy n elements of T from a host or device pointer to a host vector.
@@ -157,34 +191,10 @@ static int fetch(const T* src, size_t n, std::vector<T>& dst) {
 }
 
 static void free_universe(Universe& U) {
-    void* ptrs[] = {U.d_inv_perm, U.d_perm, U.d_sec_start, U.d_sector, U.d_qseg, U.d_sseg, U.d_B64, U.d_f64, U.d_d64, U.d_Bn1, U.d_Bn1f,
-                    U.d_mu64, U.d_B32, U.d_B32p, U.d_f32, U.d_d32, U.d_mu32, U.d_B16, U.d_Bt16, U.d_B16p, U.d_Bt16p,
-                    U.d_Cinv32, U.d_Cinv16, U.d_G32, U.d_G16, U.d_CinvF32, U.d_CinvF16};
-    for (void* p : ptrs)
-        if (p) cudaFree(p);
+    if (U.d_block) cudaFree(U.d_block);
     if (U.stream) cudaStreamDestroy(U.stream);
     U = Universe();
 }
-
-template <typename T>
-static int dalloc(Universe& U, T** p, size_t n) {
-    cudaError_t e = cudaMalloc((void**)p, n * sizeof(T));
-    if (e != cudaSuccess) {
-        set_error(std::string("cudaMalloc: ") + cudaGetErrorString(e));
-        return PRISM_ERR_ALLOCATION;
-    }
-    U.bytes += n * sizeof(T);
-    return PRISM_OK;
-}
-
-#define TRY(x)                      \
-    do {                            \
-        int rc_ = (x);              \
-        if (rc_ != PRISM_OK) {      \
-            free_universe(U);       \
-            return rc_;             \
-        }                           \
-    } while (0)
 
 static int create(const prism_universe_desc* desc, Universe& U) {
     if (!desc) { set_error("desc is NULL"); return PRISM_ERR_ARGUMENT; }
@@ -204,15 +214,12 @@ static int create(const prism_universe_desc* desc, Universe& U) {
         return PRISM_ERR_ARGUMENT;
     }
     PRISM_CUDA_TRY(cudaSetDevice(desc->device));
-    std::vector<double> B, f, d, mu;
+    std::vector<double> f, d, mu;
     std::vector<int32_t> sec;
     int rc;
-    if ((rc = fetch(desc->B, (size_t)N * K, B)) || (rc = fetch(desc->f, K, f)) ||
-        (rc = fetch(desc->d, N, d)) || (rc = fetch(desc->mu, N, mu)) ||
+    if ((rc = fetch(desc->f, K, f)) || (rc = fetch(desc->d, N, d)) || (rc = fetch(desc->mu, N, mu)) ||
         (rc = fetch(desc->sector, N, sec)))
         return rc;
-    for (size_t e = 0; e < B.size(); ++e)
-        if (!std::isfinite(B[e])) { set_error("B has a non-finite entry"); return PRISM_ERR_ARGUMENT; }
     for (int k = 0; k < K; ++k)
         if (!(f[k] > 0) || !std::isfinite(f[k])) { set_error("f must be positive and finite"); return PRISM_ERR_ARGUMENT; }
     for (int i = 0; i < N; ++i) {
@@ -234,11 +241,10 @@ static int create(const prism_universe_desc* desc, Universe& U) {
     U.sec_start.assign(S + 1, 0);
     for (int i = 0; i < N; ++i) U.sec_start[sec[i] + 1]++;
     for (int s = 0; s < S; ++s) U.sec_start[s + 1] += U.sec_start[s];
-    std::vector<double> Bs((size_t)Npad * K, 0.0), ds(Npad, 1.0), mus(Npad, 0.0);
+    std::vector<double> ds(Npad, 1.0), mus(Npad, 0.0);
     std::vector<int> secs(Npad, -1);
     for (int p = 0; p < N; ++p) {
         int i = U.perm[p];
-        std::memcpy(&Bs[(size_t)p * K], &B[(size_t)i * K], K * sizeof(double));
         ds[p] = d[i];
         mus[p] = mu[i];
         secs[p] = sec[i];
@@ -255,88 +261,103 @@ static int create(const prism_universe_desc* desc, Universe& U) {
     }
     for (int s = 0; s < S; ++s) sseg[s + 1] += sseg[s];
     U.nseg = qseg[U.nq];
-    std::vector<double> bn1(Npad, 0.0);
-    for (int p = 0; p < N; ++p)
-        for (int k = 0; k < K; ++k) bn1[p] += std::fabs(Bs[(size_t)p * K + k]);
-    std::vector<float> bn1f(bn1.begin(), bn1.end());
     cudaError_t se = cudaStreamCreateWithFlags(&U.stream, cudaStreamNonBlocking);
     if (se != cudaSuccess) { set_error(cudaGetErrorString(se)); return PRISM_ERR_CUDA; }
-    TRY(dalloc(U, &U.d_inv_perm, N));
-    TRY(dalloc(U, &U.d_perm, N));
-    TRY(dalloc(U, &U.d_sec_start, S + 1));
-    TRY(dalloc(U, &U.d_sector, Npad));
-    TRY(dalloc(U, &U.d_qseg, U.nq + 1));
-    TRY(dalloc(U, &U.d_sseg, S + 1));
-    TRY(dalloc(U, &U.d_B64, (size_t)Npad * K));
-    TRY(dalloc(U, &U.d_f64, K));
-    TRY(dalloc(U, &U.d_d64, Npad));
-    TRY(dalloc(U, &U.d_mu64, Npad));
-    TRY(dalloc(U, &U.d_Bn1, Npad));
-    TRY(dalloc(U, &U.d_Bn1f, Npad));
-    TRY(dalloc(U, &U.d_B32, (size_t)Npad * K));
-    TRY(dalloc(U, &U.d_B32p, (size_t)Npad * KMAX));
-    TRY(dalloc(U, &U.d_f32, K));
-    TRY(dalloc(U, &U.d_d32, Npad));
-    TRY(dalloc(U, &U.d_mu32, Npad));
-    TRY(dalloc(U, &U.d_B16, (size_t)Npad * K));
-    TRY(dalloc(U, &U.d_Bt16, (size_t)K * Npad));
-    TRY(dalloc(U, &U.d_B16p, (size_t)Npad * KMAX));
-    TRY(dalloc(U, &U.d_Bt16p, (size_t)KMAX * Npad));
-    TRY(dalloc(U, &U.d_Cinv32, (size_t)NRHO * K * K));
-    TRY(dalloc(U, &U.d_Cinv16, (size_t)NRHO * K * K));
-    TRY(dalloc(U, &U.d_G32, (size_t)NRHO * K * K));
-    TRY(dalloc(U, &U.d_G16, (size_t)NRHO * K * K));
-    TRY(dalloc(U, &U.d_CinvF32, (size_t)NRHO * K * K));
-    TRY(dalloc(U, &U.d_CinvF16, (size_t)NRHO * K * K));
-    auto H2D = [&](void* dst, const void* src, size_t n) {
-        return cudaMemcpy(dst, src, n, cudaMemcpyHostToDevice);
+    // One device block: what the host fills first (uploaded in one copy), then what the kernels fill,
+    // then their scratch. (27 allocations and 15 copies cost 0.5 ms here and their frees as much again.)
+    std::vector<char> image;
+    size_t off = 0;
+    std::vector<std::pair<void**, size_t>> at;
+    auto place = [&](auto** p, size_t n) {
+        at.push_back({(void**)p, off});
+        off += (n * sizeof(**p) + 255) / 256 * 256;
     };
-    if (H2D(U.d_inv_perm, U.inv_perm.data(), N * sizeof(int)) ||
-        H2D(U.d_perm, U.perm.data(), N * sizeof(int)) ||
-        H2D(U.d_sec_start, U.sec_start.data(), (S + 1) * sizeof(int)) ||
-        H2D(U.d_sector, secs.data(), Npad * sizeof(int)) ||
-        H2D(U.d_qseg, qseg.data(), (U.nq + 1) * sizeof(int)) ||
-        H2D(U.d_sseg, sseg.data(), (S + 1) * sizeof(int)) ||
-        H2D(U.d_B64, Bs.data(), Bs.size() * sizeof(double)) ||
-        H2D(U.d_f64, f.data(), K * sizeof(double)) ||
-        H2D(U.d_d64, ds.data(), Npad * sizeof(double)) ||
-        H2D(U.d_mu64, mus.data(), Npad * sizeof(double)) ||
-        H2D(U.d_Bn1, bn1.data(), Npad * sizeof(double)) ||
-        H2D(U.d_Bn1f, bn1f.data(), Npad * sizeof(float)) ||
-        H2D(U.d_f32, f32.data(), K * sizeof(float)) ||
-        H2D(U.d_d32, d32.data(), Npad * sizeof(float)) ||
-        H2D(U.d_mu32, mu32.data(), Npad * sizeof(float))) {
+    auto upload = [&](auto** p, const auto* src, size_t n) {
+        const size_t o = off;
+        place(p, n);
+        image.resize(off);
+        std::memcpy(image.data() + o, src, n * sizeof(**p));
+    };
+    int* d_bad = nullptr;
+    const int zero = 0;
+    upload(&U.d_inv_perm, U.inv_perm.data(), N);
+    upload(&U.d_perm, U.perm.data(), N);
+    upload(&U.d_sec_start, U.sec_start.data(), S + 1);
+    upload(&U.d_sector, secs.data(), Npad);
+    upload(&U.d_qseg, qseg.data(), U.nq + 1);
+    upload(&U.d_sseg, sseg.data(), S + 1);
+    upload(&U.d_f64, f.data(), K);
+    upload(&U.d_d64, ds.data(), Npad);
+    upload(&U.d_mu64, mus.data(), Npad);
+    upload(&U.d_f32, f32.data(), K);
+    upload(&U.d_d32, d32.data(), Npad);
+    upload(&U.d_mu32, mu32.data(), Npad);
+    upload(&d_bad, &zero, 1);
+    place(&U.d_B64, (size_t)Npad * K);
+    place(&U.d_Bn1, Npad);
+    place(&U.d_Bn1f, Npad);
+    place(&U.d_B32, (size_t)Npad * K);
+    place(&U.d_B32p, (size_t)Npad * KMAX);
+    place(&U.d_B16, (size_t)Npad * K);
+    place(&U.d_Bt16, (size_t)K * Npad);
+    place(&U.d_B16p, (size_t)Npad * KMAX);
+    place(&U.d_Bt16p, (size_t)KMAX * Npad);
+    place(&U.d_Cinv32, (size_t)NRHO * K * K);
+    place(&U.d_Cinv16, (size_t)NRHO * K * K);
+    place(&U.d_G32, (size_t)NRHO * K * K);
+    place(&U.d_G16, (size_t)NRHO * K * K);
+    place(&U.d_CinvF32, (size_t)NRHO * K * K);
+    place(&U.d_CinvF16, (size_t)NRHO * K * K);
+    double *G = nullptr, *raw = nullptr;
+    const bool here = on_device(desc->B, desc->device);
+    place(&G, 2 * (size_t)NRHO * K * K);
+    place(&raw, here ? 0 : (size_t)N * K);
+    if (cudaMalloc((void**)&U.d_block, off) != cudaSuccess) {
+        cudaGetLastError();
+        set_error("cudaMalloc (universe) failed");
+        free_universe(U);
+        return PRISM_ERR_ALLOCATION;
+    }
+    U.bytes = off;
+    for (auto& q : at) *q.first = U.d_block + q.second;
+    // (the default stream's copies order the upload behind what the caller queued there; they return
+    // once the host memory may be reused, and the kernels' stream is told to follow them)
+    if (cudaMemcpy(U.d_block, image.data(), image.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+        (!here && cudaMemcpy(raw, desc->B, (size_t)N * K * sizeof(double), cudaMemcpyDefault) != cudaSuccess) ||
+        cudaStreamSynchronize(0) != cudaSuccess) {
+        cudaGetLastError();
         set_error("universe upload failed");
         free_universe(U);
         return PRISM_ERR_CUDA;
     }
-    {
-        size_t n = (size_t)Npad * K;
-        cudaMemsetAsync(U.d_B32p, 0, (size_t)Npad * KMAX * 4, U.stream);
-        cudaMemsetAsync(U.d_B16p, 0, (size_t)Npad * KMAX * 2, U.stream);
-        cudaMemsetAsync(U.d_Bt16p, 0, (size_t)KMAX * Npad * 2, U.stream);
-        k_convert_B<<<(unsigned)cdiv64(n, 256), 256, 0, U.stream>>>(U.d_B64, Npad, K, U.d_B32, U.d_B32p, U.d_B16, U.d_Bt16,
-                                                                      U.d_B16p, U.d_Bt16p);
-        double* G = nullptr;
-        if (cudaMalloc(&G, (size_t)NRHO * K * K * sizeof(double)) != cudaSuccess) {
-            set_error("cudaMalloc (Gram scratch) failed");
-            free_universe(U);
-            return PRISM_ERR_ALLOCATION;
-        }
-        dim3 grid(NRHO, cdiv(K, 8));
-        k_gram<float><<<grid, 256, 0, U.stream>>>(U.d_B32, U.d_d32, N, K, G);
-        k_cinv<<<NRHO, 64, 0, U.stream>>>(G, U.d_f64, K, U.d_Cinv32, 0, U.d_G32);
-        k_cinv<<<NRHO, 64, 0, U.stream>>>(G, U.d_f64, K, U.d_CinvF32, 1, nullptr);
-        k_gram<__nv_bfloat16><<<grid, 256, 0, U.stream>>>(U.d_B16, U.d_d32, N, K, G);
-        k_cinv<<<NRHO, 64, 0, U.stream>>>(G, U.d_f64, K, U.d_Cinv16, 0, U.d_G16);
-        k_cinv<<<NRHO, 64, 0, U.stream>>>(G, U.d_f64, K, U.d_CinvF16, 1, nullptr);
-        cudaError_t e = cudaStreamSynchronize(U.stream);
-        cudaFree(G);
-        if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) {
-            set_error(std::string("universe setup kernels failed: ") + cudaGetErrorString(e));
-            free_universe(U);
-            return PRISM_ERR_CUDA;
-        }
+    ConvArgs CA;
+    CA.raw = here ? desc->B : raw;
+    CA.perm = U.d_perm; CA.N = N; CA.Npad = Npad; CA.K = K;
+    CA.B64 = U.d_B64; CA.B32 = U.d_B32; CA.B32p = U.d_B32p;
+    CA.B16 = U.d_B16; CA.Bt16 = U.d_Bt16; CA.B16p = U.d_B16p; CA.Bt16p = U.d_Bt16p;
+    CA.Bn1 = U.d_Bn1; CA.Bn1f = U.d_Bn1f; CA.bad = d_bad;
+    k_convert_B<<<(unsigned)cdiv64((int64_t)Npad * 32, 256), 256, 0, U.stream>>>(CA);
+    k_gram<<<dim3(NRHO, cdiv(K, 8), 2), 256, 0, U.stream>>>(U.d_B32, U.d_B16, U.d_d32, N, K, G);
+    CinvArgs IA;
+    IA.G = G; IA.f = U.d_f64; IA.K = K;
+    IA.out[0] = U.d_Cinv32; IA.out[1] = U.d_Cinv16; IA.out[2] = U.d_CinvF32; IA.out[3] = U.d_CinvF16;
+    IA.G_out[0] = U.d_G32; IA.G_out[1] = U.d_G16;
+    const int smem = 2 * K * (K + 1) * (int)sizeof(double);
+    cudaFuncSetAttribute(k_cinv, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    k_cinv<<<dim3(NRHO, 4), 256, smem, U.stream>>>(IA);
+    int bad = 0;
+    cudaError_t e = cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, U.stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(U.stream);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) {
+        set_error(std::string("universe setup kernels failed: ") + cudaGetErrorString(e));
+        free_universe(U);
+        return PRISM_ERR_CUDA;
+    }
+    if (bad) {
+        set_error("B has a non-finite entry");
+        free_universe(U);
+        return PRISM_ERR_ARGUMENT;
     }
     return PRISM_OK;
 }
