@@ -250,6 +250,7 @@ extern "C" int prism_polish_noalloc(prism_universe* uh, const prism_batch* b, co
     const size_t MN = (size_t)M * Npad;
     // carve the static array
     NaCarve cv{g_na_base[U.device]};
+    // what has to be zero at the start first, so that one memset clears it
     double* W0 = cv.take<double>(MN); double* LO = cv.take<double>(MN);
     double* UP = cv.take<double>(MN); double* Cc = cv.take<double>(MN);
     double* W = cv.take<double>(MN);
@@ -257,6 +258,13 @@ extern "C" int prism_polish_noalloc(prism_universe* uh, const prism_batch* b, co
     float* W0f = cv.take<float>(MN); float* LOf = cv.take<float>(MN);
     float* UPf = cv.take<float>(MN); float* Cf = cv.take<float>(MN);
     int* member = cv.take<int>(MN);
+    double* lam = cv.take<double>((size_t)M * S);
+    double* nu = cv.take<double>(M); double* theta = cv.take<double>(M);
+    int* done = cv.take<int>(M); int* skip = cv.take<int>(M);
+    int* status = cv.take<int>(M); int* iters = cv.take<int>(M);
+    double* diag = cv.take<double>((size_t)M * PRISM_NDIAG);
+    int* err = cv.take<int>(4);
+    const size_t zeroed = cv.used;
     int8_t* stt = cv.take<int8_t>(MN);
     double* s_w0 = cv.take<double>(nnz); double* s_lo = cv.take<double>(nnz);
     double* s_up = cv.take<double>(nnz); double* s_tc = cv.take<double>(nnz);
@@ -264,14 +272,10 @@ extern "C" int prism_polish_noalloc(prism_universe* uh, const prism_batch* b, co
     int32_t* s_idx = cv.take<int32_t>(nnz);
     int64_t* s_off = cv.take<int64_t>(M + 1);
     double* blo = cv.take<double>((size_t)M * S); double* bhi = cv.take<double>((size_t)M * S);
-    double* lam = cv.take<double>((size_t)M * S);
     int* wband = cv.take<int>((size_t)M * S);
     float* eta_hi = cv.take<float>((size_t)M * S); float* eta_lo = cv.take<float>((size_t)M * S);
-    double* tau = cv.take<double>(M); double* nu = cv.take<double>(M); double* theta = cv.take<double>(M);
-    int* wcap = cv.take<int>(M); int* done = cv.take<int>(M); int* skip = cv.take<int>(M);
-    int* status = cv.take<int>(M); float* nu_f = cv.take<float>(M); float* theta_f = cv.take<float>(M);
-    int* iters = cv.take<int>(M);
-    double* diag = cv.take<double>((size_t)M * PRISM_NDIAG);
+    double* tau = cv.take<double>(M);
+    int* wcap = cv.take<int>(M); float* nu_f = cv.take<float>(M); float* theta_f = cv.take<float>(M);
     const int FMAX = std::min(N, NA_FMAX);
     int* Fl = cv.take<int>((size_t)M * FMAX); int* NZl = cv.take<int>((size_t)M * FMAX);
     double* Fsig = cv.take<double>((size_t)M * FMAX);
@@ -283,7 +287,6 @@ extern "C" int prism_polish_noalloc(prism_universe* uh, const prism_batch* b, co
     double* fhmax = cv.take<double>(M);
     int* ndep = cv.take<int>(M);
     int* pending = cv.take<int>(4);
-    int* err = cv.take<int>(4);
     if (cv.overflow) return na_fail(PRISM_ERR_ARGUMENT, "prism_polish_noalloc: request exceeds the static scratch");
     // stage the inputs (host pointers are copied into the scratch, device pointers used in place)
     auto stage = [&](const void* src, void* dst, size_t bytes) -> const void* {
@@ -305,17 +308,8 @@ extern "C" int prism_polish_noalloc(prism_universe* uh, const prism_batch* b, co
     A.W0 = W0; A.LO = LO; A.UP = UP; A.C = Cc; A.Z = Z; A.member = member; A.err = err;
     A.W0f = W0f; A.LOf = LOf; A.UPf = UPf; A.Cf = Cf;
     // the array keeps the previous call's contents: clear everything read before written
-    cudaMemsetAsync(W0, 0, MN * 8, st); cudaMemsetAsync(LO, 0, MN * 8, st);
-    cudaMemsetAsync(UP, 0, MN * 8, st); cudaMemsetAsync(Cc, 0, MN * 8, st);
-    cudaMemsetAsync(W, 0, MN * 8, st); cudaMemsetAsync(Z, 0, MN * 4, st);
-    cudaMemsetAsync(W0f, 0, MN * 4, st); cudaMemsetAsync(LOf, 0, MN * 4, st);
-    cudaMemsetAsync(UPf, 0, MN * 4, st); cudaMemsetAsync(Cf, 0, MN * 4, st);
-    cudaMemsetAsync(member, 0, MN * 4, st); cudaMemsetAsync(err, 0, 16, st);
-    cudaMemsetAsync(done, 0, M * 4, st); cudaMemsetAsync(skip, 0, M * 4, st);
-    cudaMemsetAsync(status, 0, M * 4, st); cudaMemsetAsync(iters, 0, M * 4, st);
-    cudaMemsetAsync(diag, 0, (size_t)M * PRISM_NDIAG * 8, st);
-    cudaMemsetAsync(nu, 0, M * 8, st); cudaMemsetAsync(theta, 0, M * 8, st);
-    cudaMemsetAsync(lam, 0, (size_t)M * S * 8, st);
+    // (one memset of what lies together: 20 of them took 50 us of a 384 us call for eight accounts)
+    cudaMemsetAsync(W0, 0, zeroed, st);
     cudaMemcpyAsync(blo, b->band_lo, (size_t)M * S * 8, cudaMemcpyDefault, st);
     cudaMemcpyAsync(bhi, b->band_hi, (size_t)M * S * 8, cudaMemcpyDefault, st);
     if (b->turnover_cap) cudaMemcpyAsync(tau, b->turnover_cap, M * 8, cudaMemcpyDefault, st);
