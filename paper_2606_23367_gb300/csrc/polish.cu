@@ -1395,12 +1395,12 @@ void launch_classify(const PolDev& P, cudaStream_t st) { k_classify<<<P.M, PB, 0
 
 // Up to `rounds` active-set rounds for every account not yet settled, in one launch: blocks of 256 threads,
 // two to an SM, or of 512 when there are no more accounts than SMs (the passes over all entries then
-// take half the time).
-void launch_polish(const PolDev& P, int rounds, cudaStream_t st) {
+// take half the time). accounts: how many are not settled (0: all).
+void launch_polish(const PolDev& P, int rounds, cudaStream_t st, int accounts) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (P.M <= sms) {
+    if ((accounts > 0 ? accounts : P.M) <= sms) {
         cudaFuncSetAttribute(k_polish<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PolishShared));
         k_polish<512><<<P.M, 512, sizeof(PolishShared), st>>>(P, rounds);
     } else {

@@ -84,7 +84,7 @@ struct PolDev {
 
 size_t polish_smem_bytes();
 void launch_classify(const PolDev& P, cudaStream_t st);
-void launch_polish(const PolDev& P, int rounds, cudaStream_t st);
+void launch_polish(const PolDev& P, int rounds, cudaStream_t st, int accounts = 0);
 void launch_fallback(const PolDev& P, cudaStream_t st);
 void launch_finish_status(const PolDev& P, double eps, cudaStream_t st);
 // Per-entry active-set flags of the polished solution for the adjoint:

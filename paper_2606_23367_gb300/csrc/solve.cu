@@ -3,11 +3,13 @@
 // Call structure (one call = one book of accounts, Fig. 2 public solver call):
 //   1. validate and pack the ragged FP64 inputs into a sector-sorted M x Npad
 //      device layout (FP64 copies for the polish, FP32 copies for the iterations);
-//      lot data become per-entry piecewise-linear cost tables;
+//      lot data become per-entry piecewise-linear cost tables (built on the device);
 //   2. closed-form capacity test per account (budget, box and bands admit a point);
 //      accounts that fail get NO_FEASIBLE_RETURN;
-//   3. ADMM iterations, check_every at a time, captured once in a CUDA graph and
-//      replayed until every account has converged or hit its cap;
+//   3. ADMM iterations: account-resident, all of an account's iterations in one launch
+//      (acct_route chooses), or batched over the book, check_every at a time, captured once
+//      in a CUDA graph and replayed until every account has converged or hit its cap, the
+//      last few accounts account-resident (few_fit);
 //   4. FP64 polish rounds and certification; accounts the polish cannot settle go
 //      back to the iterations with a tighter target, then fall back to the
 //      projected iterate (FEASIBLE_NONCERTIFIED when it passes the gates);
@@ -587,6 +589,13 @@ struct AcctClass {
     AcctShape shape;
 };
 
+static int sm_count() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(1, sms);
+}
+
 // Time of one iteration of the whole book, us, as measured at 500 to 10,000 assets, 16 to 64 factors and
 // 16 to 500 accounts. Account-resident: 4.5 for the chain of reductions, 2.5 more when it crosses a
 // cluster, and the products with the CTA's rows; times the waves of clusters.
@@ -603,18 +612,19 @@ static double batched_iteration_us(int M, int N, bool bf16, bool staged) {
     return (staged ? 60.0 : 30.0) + (bf16 ? 9e-6 : 3e-5) * M * N;
 }
 
+// Whether the options leave the form of the iterations open: one that names a form of the batched
+// kernels keeps the book on them, and so does the failure-path test of their tensor-core waits.
+static bool open_form(const prism_solve_opts& o) {
+    return !(o.fold_products || o.xupdate_form || o.chains || o.g2_sets || !o.fuse_prox || o.ragged_layout == 1) &&
+           !std::getenv("PRISM_TEST_STALLED_WAIT_NS");
+}
+
 static bool acct_route(const prism_solve_opts& o, bool plain, bool fp64, bool bf16, bool ragged, int M, int N, int K,
                        bool pw, bool tilt, bool fac, bool cap, const std::vector<int64_t>& offs, std::vector<AcctClass>& classes,
                        std::vector<int>& order) {
-    // an option that names a form of the batched kernels keeps the book on them, and so does the
-    // failure-path test of their tensor-core waits
-    if (o.fold_products || o.xupdate_form || o.chains || o.g2_sets || !o.fuse_prox || o.ragged_layout == 1) return false;
-    if (std::getenv("PRISM_TEST_STALLED_WAIT_NS")) return false;
+    if (!open_form(o)) return false;
     const int bytes = fp64 ? 8 : (bf16 ? 2 : 4);
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    sms = std::max(1, sms);
+    const int sms = sm_count();
     classes.clear();
     order.clear();
     double us = 0.0;
@@ -798,7 +808,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         // state and input copies for accounts too large for shared memory
         const size_t np = packed ? (size_t)nnz : 0;
         PK.plist = A.take<int>(lists ? (size_t)nnz : 0); PK.psec = A.take<int>(lists ? (size_t)M * (S + 1) : 0);
-        PK.order = A.take<int>(lists ? M : 0); PK.queue = A.take<int>(4);
+        PK.order = A.take<int>(M); PK.queue = A.take<int>(4);
         t0_dev = A.take<unsigned long long>(1);
         inbox = A.take<char>(SolveCache::BOX);
         PK.z = A.take<float>(np); PK.y = A.take<float>(np); PK.X = A.take<float>(np);
@@ -1197,6 +1207,92 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         SC.prof.run(PRISM_K_OTHER, 1, s, [&] { launch_classify(PB2, s); });
         SC.prof.run(PRISM_K_POLISH, 1, s, [&] { launch_polish(PB2, rounds, s); });
     };
+    AcctArgs<float> AF;
+    AcctArgs<double> AD;
+    // the few accounts that a batched book sends back to the iterations go on account-resident
+    const AcctShape again = (!acct && !fp64 && !packed && !b->asset_idx && open_form(*o))
+                                ? acct_shape(N, K, batched_mode_bf16 ? 2 : 4, false, BD.has_fac, has_pw) : AcctShape();
+    if (acct || again.E) {
+        auto fill = [&](auto& A) {
+            A.M = M; A.N = N; A.Npad = Npad; A.K = K; A.S = S;
+            A.sec_start = U.d_sec_start;
+            A.pw_idx = pwidx; A.pw_nbp = BD.pw_nbp;
+            A.nu = D.nu; A.eta_hi = D.eta_hi; A.eta_lo = D.eta_lo; A.theta = D.theta; A.zf = D.z;
+            A.rho_idx = D.rho_idx; A.iters = D.iters; A.active = D.active; A.status = D.status;
+            if (b->asset_idx) { A.plist = PK.plist; A.poff = PA.offsets; A.psec = PK.psec; }
+            if (BD.has_fac) A.sflag = D.sflag;
+            A.t0 = t0_dev;
+            // With lots or a cap the polish can lose its way from a start a few places off, and one such
+            // account costs it eight rounds on hundreds of free entries: 8-11 ms of a 200 x 1,924 book
+            // against 0.6 when every account first keeps its places for 12 iterations (ADMM 1.6 -> 2.2
+            // ms). Books without them gain nothing (100 x 5,000 x 48: 1.3 -> 2.3 against 0.67 -> 0.47).
+            A.settle = (has_lots || BD.has_cap) ? 12 : 0;
+            A.alpha = o->alpha; A.eps = o->eps_admm;
+            A.max_iter = o->max_iter; A.min_iter = o->min_iter; A.adapt_every = D.adapt_every;
+        };
+        fill(AF);
+        fill(AD);
+        if (batched_mode_bf16) AF.B16p = U.d_B16p; else AF.B32p = U.d_B32p;
+        AF.f = U.d_f32; AF.d = U.d_d32; AF.mu = U.d_mu32;
+        if (!b->asset_idx) { AF.Cinv = D.Cinv; AF.G = D.G; }   // (of the split-off factor block when there is one)
+        AF.w0 = BD.w0f; AF.lo = BD.lof; AF.up = BD.upf; AF.c = BD.cf;
+        AF.pw_bp = BD.pw_bpf; AF.pw_sl = BD.pw_slf;
+        AF.band_lo = BD.band_lof; AF.band_hi = BD.band_hif;
+        AF.z = D.z; AF.y = D.y;
+        AF.tilt = P.tiltf; AD.tilt = P.tilt;
+        if (BD.has_cap) AF.tau = BD.tauf;
+        if (BD.has_fac) { AF.flo = BD.flof; AF.fhi = BD.fhif; AF.s = D.s; AF.ys = D.ys; }
+        AD.B64 = U.d_B64; AD.f = U.d_f64; AD.d = U.d_d64; AD.mu = U.d_mu64;
+        AD.w0 = BD.w0; AD.lo = BD.lo; AD.up = BD.up; AD.c = BD.c;
+        AD.pw_bp = BD.pw_bp; AD.pw_sl = BD.pw_sl;
+        AD.band_lo = BD.band_lo; AD.band_hi = BD.band_hi;
+        AD.z = P64.z; AD.y = P64.y;
+        if (BD.has_cap) AD.tau = BD.tau;
+        if (BD.has_fac) { AD.flo = BD.flo; AD.fhi = BD.fhi; AD.s = P64.s_state; AD.ys = P64.ys_state; }
+    }
+    // the accounts' iterations, one launch per class of sizes (side by side on the chains' streams)
+    auto set_budget = [&]() {                         // (from t0, which the device took a little after the call began)
+        if (o->time_budget_s > 0)
+            AF.budget_ns = AD.budget_ns = (unsigned long long)(std::min(o->time_budget_s, 1e9) * 1e9) + 1;
+    };
+    auto run_acct = [&](int resume, double eps, int max_iter) {
+        set_budget();
+        AF.resume = AD.resume = resume;
+        AF.eps = (float)eps; AD.eps = eps;
+        AF.max_iter = AD.max_iter = max_iter;
+        const int nstream = SC.chains_ok && !SC.prof.on ? std::min<int>(SolveCache::MAXCH, (int)classes.size()) : 1;
+        SC.prof.run(PRISM_K_BLOCK, (int)classes.size(), st, [&] {
+            if (nstream > 1) cudaEventRecord(SC.ev_fork, st);
+            for (int c = 1; c < nstream; ++c) cudaStreamWaitEvent(SC.chst[c - 1], SC.ev_fork, 0);
+            for (size_t c = 0; c < classes.size(); ++c) {
+                const AcctClass& q = classes[c];
+                cudaStream_t s = c % nstream ? SC.chst[c % nstream - 1] : st;
+                AF.order = AD.order = b->asset_idx ? PK.order + q.first : nullptr;
+                if (fp64) launch_acct_admm(AD, q.shape, q.count, s);
+                else launch_acct_admm(AF, q.shape, q.count, s);
+            }
+            for (int c = 1; c < nstream; ++c) {
+                cudaEventRecord(SC.ev_join[c - 1], SC.chst[c - 1]);
+                cudaStreamWaitEvent(st, SC.ev_join[c - 1], 0);
+            }
+        });
+    };
+    // A batched book with only a few accounts left to iterate goes on account-resident once their CTAs
+    // fit on the SMs side by side: the chain of the batched kernels costs 21-25 us an iteration however
+    // few accounts are left and runs on to the end of its chunk. One to three accounts of 500 x 10,000 x
+    // 64 that the polish sends back: 2.3-3.1 ms on the chain, 0.9-1.6 so (of calls of 6.0 ms without).
+    auto few_fit = [&](int n) { return again.E && n > 0 && n * again.cluster <= sm_count(); };
+    auto run_few = [&](const int* act, double eps, int max_iter) {
+        order_h.clear();
+        for (int a = 0; a < M; ++a) if (act[a]) order_h.push_back(a);
+        cudaMemcpyAsync(PK.order, order_h.data(), order_h.size() * 4, cudaMemcpyHostToDevice, st);
+        AF.resume = 1;
+        AF.eps = (float)eps;
+        AF.max_iter = max_iter;
+        AF.order = PK.order;
+        set_budget();
+        SC.prof.run(PRISM_K_BLOCK, 1, st, [&] { launch_acct_admm(AF, again, (int)order_h.size(), st); });
+    };
     auto admm_loop = [&](int iter_budget, bool overlap) -> int {
         int done_iters = 0;
         if (D.needP) {
@@ -1257,6 +1353,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
                 }
             }
             if (SC.pinned[0] == 0) break;
+            if (!overlap && few_fit(SC.pinned[0])) { run_few(SC.hact, D.eps_admm, D.max_iter); break; }
             if (o->time_budget_s > 0) {
                 double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t_call0).count();
                 if (el > o->time_budget_s) break;
@@ -1268,72 +1365,6 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     // to have settled (its moves set the streaming form's margin) to keep its candidate lists short
     const bool blockwise = acct || fp64 || packed;   // every iteration inside a per-account kernel
     const int cold = (D.stream_prox && !blockwise) ? std::min(std::max(0, o->stream_after), o->max_iter) : 0;
-    AcctArgs<float> AF;
-    AcctArgs<double> AD;
-    if (acct) {
-        auto fill = [&](auto& A) {
-            A.M = M; A.N = N; A.Npad = Npad; A.K = K; A.S = S;
-            A.sec_start = U.d_sec_start;
-            A.pw_idx = pwidx; A.pw_nbp = BD.pw_nbp;
-            A.nu = D.nu; A.eta_hi = D.eta_hi; A.eta_lo = D.eta_lo; A.theta = D.theta; A.zf = D.z;
-            A.rho_idx = D.rho_idx; A.iters = D.iters; A.active = D.active; A.status = D.status;
-            if (b->asset_idx) { A.plist = PK.plist; A.poff = PA.offsets; A.psec = PK.psec; }
-            if (BD.has_fac) A.sflag = D.sflag;
-            A.t0 = t0_dev;
-            // With lots or a cap the polish can lose its way from a start a few places off, and one such
-            // account costs it eight rounds on hundreds of free entries: 8-11 ms of a 200 x 1,924 book
-            // against 0.6 when every account first keeps its places for 12 iterations (ADMM 1.6 -> 2.2
-            // ms). Books without them gain nothing (100 x 5,000 x 48: 1.3 -> 2.3 against 0.67 -> 0.47).
-            A.settle = (has_lots || BD.has_cap) ? 12 : 0;
-            A.alpha = o->alpha; A.eps = o->eps_admm;
-            A.max_iter = o->max_iter; A.min_iter = o->min_iter; A.adapt_every = D.adapt_every;
-        };
-        fill(AF);
-        fill(AD);
-        if (batched_mode_bf16) AF.B16p = U.d_B16p; else AF.B32p = U.d_B32p;
-        AF.f = U.d_f32; AF.d = U.d_d32; AF.mu = U.d_mu32;
-        if (!b->asset_idx) { AF.Cinv = D.Cinv; AF.G = D.G; }   // (of the split-off factor block when there is one)
-        AF.w0 = BD.w0f; AF.lo = BD.lof; AF.up = BD.upf; AF.c = BD.cf;
-        AF.pw_bp = BD.pw_bpf; AF.pw_sl = BD.pw_slf;
-        AF.band_lo = BD.band_lof; AF.band_hi = BD.band_hif;
-        AF.z = D.z; AF.y = D.y;
-        AF.tilt = P.tiltf; AD.tilt = P.tilt;
-        if (BD.has_cap) AF.tau = BD.tauf;
-        if (BD.has_fac) { AF.flo = BD.flof; AF.fhi = BD.fhif; AF.s = D.s; AF.ys = D.ys; }
-        AD.B64 = U.d_B64; AD.f = U.d_f64; AD.d = U.d_d64; AD.mu = U.d_mu64;
-        AD.w0 = BD.w0; AD.lo = BD.lo; AD.up = BD.up; AD.c = BD.c;
-        AD.pw_bp = BD.pw_bp; AD.pw_sl = BD.pw_sl;
-        AD.band_lo = BD.band_lo; AD.band_hi = BD.band_hi;
-        AD.z = P64.z; AD.y = P64.y;
-        if (BD.has_cap) AD.tau = BD.tau;
-        if (BD.has_fac) { AD.flo = BD.flo; AD.fhi = BD.fhi; AD.s = P64.s_state; AD.ys = P64.ys_state; }
-    }
-    // the accounts' iterations, one launch per class of sizes (side by side on the chains' streams)
-    auto run_acct = [&](int resume, double eps, int max_iter) {
-        if (o->time_budget_s > 0) {
-            const double left = o->time_budget_s - std::chrono::duration<double>(std::chrono::steady_clock::now() - t_call0).count();
-            AF.budget_ns = AD.budget_ns = (unsigned long long)(std::min(std::max(left, 0.0), 1e9) * 1e9) + 1;
-        }
-        AF.resume = AD.resume = resume;
-        AF.eps = (float)eps; AD.eps = eps;
-        AF.max_iter = AD.max_iter = max_iter;
-        const int nstream = SC.chains_ok && !SC.prof.on ? std::min<int>(SolveCache::MAXCH, (int)classes.size()) : 1;
-        SC.prof.run(PRISM_K_BLOCK, (int)classes.size(), st, [&] {
-            if (nstream > 1) cudaEventRecord(SC.ev_fork, st);
-            for (int c = 1; c < nstream; ++c) cudaStreamWaitEvent(SC.chst[c - 1], SC.ev_fork, 0);
-            for (size_t c = 0; c < classes.size(); ++c) {
-                const AcctClass& q = classes[c];
-                cudaStream_t s = c % nstream ? SC.chst[c % nstream - 1] : st;
-                AF.order = AD.order = b->asset_idx ? PK.order + q.first : nullptr;
-                if (fp64) launch_acct_admm(AD, q.shape, q.count, s);
-                else launch_acct_admm(AF, q.shape, q.count, s);
-            }
-            for (int c = 1; c < nstream; ++c) {
-                cudaEventRecord(SC.ev_join[c - 1], SC.chst[c - 1]);
-                cudaStreamWaitEvent(st, SC.ev_join[c - 1], 0);
-            }
-        });
-    };
     if (acct) {
         if (b->asset_idx)
             SC.prof.run(PRISM_K_OTHER, 1, st, [&] {
@@ -1395,10 +1426,10 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     int n_rounds_run = 0, n_retried = 0;
     // all active-set rounds of every account in one launch; each block stops when settled (one
     // launch per round measured slower: each launch waits for its slowest block)
-    auto polish_rounds = [&](bool last) -> int {
+    auto polish_rounds = [&](bool last, int accounts) -> int {
         ++n_rounds_run;
         P.retry = !last;
-        SC.prof.run(PRISM_K_POLISH, 1, st, [&] { launch_polish(P, rounds, st); });
+        SC.prof.run(PRISM_K_POLISH, 1, st, [&] { launch_polish(P, rounds, st, accounts); });
         return 0;
     };
     if (pol_gen > 0) {
@@ -1411,7 +1442,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         polish_batch(0, st);
     } else {
         SC.prof.run(PRISM_K_OTHER, 1, st, [&] { launch_classify(P, st); });
-        if (polish_rounds(false) < 0) { set_error("polish failed"); return PRISM_ERR_CUDA; }
+        if (polish_rounds(false, M) < 0) { set_error("polish failed"); return PRISM_ERR_CUDA; }
     }
     for (int retry = 0; retry < 2; ++retry) {
         SC.prof.run(PRISM_K_OTHER, 1, st, [&] { k_unsettled<<<1, 1024, 0, st>>>(M, P.skip, P.done, D.status, err + 3); });
@@ -1442,8 +1473,11 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         PRISM_CUDA_TRY(cudaMemcpyAsync(P.done, done.data(), M * 4, cudaMemcpyHostToDevice, st));
         PRISM_CUDA_TRY(cudaStreamSynchronize(st));
         int more = 0;
+        const int sent_back = n_retry;
         if (acct) {
             run_acct(1, o->eps_admm * (retry == 0 ? 0.1 : 0.01), o->max_iter * (retry + 2));
+        } else if (few_fit(n_retry)) {
+            run_few(act.data(), o->eps_admm * (retry == 0 ? 0.1 : 0.01), o->max_iter * (retry + 2));
         } else if (fp64) {
             // continue the FP64 iterations of the accounts sent back, to a tighter target
             BlkArgs<double> R = P64;
@@ -1468,7 +1502,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         if (more < 0) { set_error("ADMM retry failed"); return PRISM_ERR_CUDA; }
         total_iters += more;
         SC.prof.run(PRISM_K_OTHER, 1, st, [&] { launch_classify(P, st); });
-        if (polish_rounds(retry == 1) < 0) { set_error("polish failed"); return PRISM_ERR_CUDA; }
+        if (polish_rounds(retry == 1, sent_back) < 0) { set_error("polish failed"); return PRISM_ERR_CUDA; }
     }
     if (std::getenv("PRISM_DEBUG_STATS"))
         std::fprintf(stderr, "prism stats: polish rounds %d, accounts sent back to the iterations %d\n", n_rounds_run,

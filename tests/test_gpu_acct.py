@@ -93,3 +93,21 @@ def test_time_budget_stops_every_account():
     assert int(res["iters"].max()) == 1
     assert set(res["status"].tolist()) <= {prism.PRISM_TIMEOUT, prism.PRISM_CERTIFIED}
     assert (res["status"] == prism.PRISM_TIMEOUT).any()
+
+
+@pytest.mark.parametrize("rounds", [None, 3])
+@pytest.mark.parametrize("kind,N,M,mode", [(1, 3000, 400, prism.PRISM_BATCHED_BF16), (1, 3000, 400, prism.PRISM_BATCHED_FP32),
+                                           (3, 2000, 600, prism.PRISM_BATCHED_BF16)])
+def test_a_batched_book_hands_its_last_accounts_over(kind, N, M, mode, rounds):
+    # more accounts than the account-resident form is faster for: batched, until few iterate on or few
+    # come back from a polish cut short, and the weights of the batched kernels alone
+    uni, batch = make_workload(kind, N=N, K=64, S=20, M=M)
+    opts = dict(precision=mode, check_every=5, **({} if rounds is None else dict(polish_rounds=rounds)))
+    new, old = gpu_solve(uni, batch, **opts), gpu_solve(uni, batch, chains=1, **opts)
+    block = prism.KERNEL_CLASSES.index("block")
+    assert new["kernel_launches"][block] >= 1 and old["kernel_launches"][block] == 0
+    assert new["kernel_launches"][prism.KERNEL_CLASSES.index("gemm_P")] > 0
+    sure = old["status"] == prism.PRISM_CERTIFIED
+    assert sure.any() and np.all(new["status"][sure] == prism.PRISM_CERTIFIED)
+    acct = np.repeat(sure, np.diff(batch.offsets))
+    assert float(np.max(np.abs(new["w"] - old["w"])[acct])) <= 1e-9
