@@ -631,13 +631,14 @@ def run_gpu(args, dist, rank, world, local_rank):
            "prox": M * N if fused else N * it_sum / max(1, n_launch["prox"])}
     if fused:
         ent["xprox"] = prof["stream_entries"] / kl[ix]
-    if n_launch["block"] > 0:
+    if n_launch["block"] > 0 and n_launch["gemm_P"] == 0:
+        # (a batched book hands only its last accounts over: those launches have no figure here)
         # the per-account kernel runs every iteration of its accounts in one launch: the
         # account's own names times its iterations
         own = np.diff(batch.offsets).astype(np.float64)
         ent["block"] = float((own * iters).sum()) / n_launch["block"]
     alg = {n: ALG_BYTES[n] * ent[n] for n in ent}
-    dom = max(step_ms, key=lambda n: step_ms[n])
+    dom = max(ent, key=lambda n: step_ms[n])
     avg_ms = step_ms[dom] / max(1, n_launch[dom])
     peaks = {}
     try:
@@ -648,7 +649,7 @@ def run_gpu(args, dist, rank, world, local_rank):
     achieved = alg[dom] / (avg_ms / 1000.0) / 1e9
     persistent = opts.get("xupdate_form", 0) == 0 and not opts.get("fold_products", 0)
     kernel_of = {"gemm_P": "k_tc_gemm_P", "gemm_x": "k_tc_gemm_x", "prox": "k_prox_stream / k_prox_smem",
-                 "xprox": "k_tc_xprox_pers" if persistent else "k_tc_xprox", "block": "k_block_admm"}
+                 "xprox": "k_tc_xprox_pers" if persistent else "k_tc_xprox", "block": "k_acct_admm / k_block_admm"}
     # the whole iteration: the method's bytes of every account-iteration of the step over the
     # step's device time (setup, polish and certification included in the time)
     iter_bytes = METHOD_BYTES * N * float(iters.sum())

@@ -129,7 +129,8 @@ typedef struct {
     double  eps_admm;         /* ADMM residual target before the polish (default 5e-4) */
     double  rho0;             /* initial ADMM penalty (default 3.0) */
     double  alpha;            /* over-relaxation (default 1.5) */
-    double  time_budget_s;    /* wall-clock ceiling for the call (<= 0: none) */
+    double  time_budget_s;    /* wall-clock ceiling for the call (<= 0: none); looked at after every
+                                 captured chunk of iterations, account-resident after every iteration */
     int32_t max_iter;         /* ADMM iteration cap per account (default 4000) */
     int32_t check_every;      /* iterations per captured graph launch (default 20) */
     int32_t min_iter;         /* iterations before a convergence test may stop an account */
@@ -142,6 +143,11 @@ typedef struct {
     double  polish_overlap;   /* accounts that stop iterating are polished beside the iterations once
                                  fewer than this fraction of the book still iterates (0 = never:
                                  the whole book is polished after the iterations; default 0) */
+    /* Books whose accounts fit run account-resident where that is estimated to be the faster: every
+     * iteration of an account in one launch, its rows of B in shared memory (up to 16,384 names). The
+     * options chains, fuse_prox = 0, g2_sets, fold_products, xupdate_form and ragged_layout = 1 each
+     * name a form of the batched kernels and keep a book on them; check_every, stream_after, use_graph
+     * and polish_overlap have no effect on account-resident books. */
     int32_t chains;           /* fused iterations: the book is cut into this many account ranges
                                  (multiples of 128) that iterate independently on their own
                                  streams; 0 = one with the persistent x-update (xupdate_form 0),
@@ -154,10 +160,12 @@ typedef struct {
     void*   cuda_stream;      /* cudaStream_t to run on (NULL = the library's own stream) */
     int32_t ragged_layout;    /* books with asset_idx in the batched modes: 1 = dense-masked over the
                                  universe (every product over all N positions, non-members pinned
-                                 at 0); 2 = packed (each account's own names only, one persistent
-                                 launch of per-account blocks with the account's own capacitance);
-                                 0 = dense-masked (the faster of the two on the workloads measured;
-                                 prism_autotune times both for a book) (default 0) */
+                                 at 0); 2 = packed (each account's own names only, with the
+                                 account's own capacitance: account-resident, see chains, while the
+                                 largest account fits, else one persistent launch of per-account
+                                 blocks); 0 = packed account-resident where that is estimated to be
+                                 the faster, else dense-masked (prism_autotune times the layouts for
+                                 a book) (default 0) */
     int32_t g2_sets;          /* tile shape of the tensor-core product B'X: clusters of 8 CTAs per
                                  128-account tile along the assets, each CTA summing an asset chunk
                                  of N / (8 g2_sets) (rounded up to 64); 0 = about one CTA per SM
