@@ -111,3 +111,15 @@ def test_a_batched_book_hands_its_last_accounts_over(kind, N, M, mode, rounds):
     assert sure.any() and np.all(new["status"][sure] == prism.PRISM_CERTIFIED)
     acct = np.repeat(sure, np.diff(batch.offsets))
     assert float(np.max(np.abs(new["w"] - old["w"])[acct])) <= 1e-9
+
+
+@pytest.mark.parametrize("mode", [prism.PRISM_BATCHED_BF16, prism.PRISM_BATCHED_FP32])
+@pytest.mark.parametrize("seed", [101, 102])
+def test_a_band_edge_that_the_bounds_imply_has_no_multiplier(mode, seed):
+    # long-only books with band floors of 0: the floor holds by the entries' own bounds, so that its
+    # multiplier, which a sector sold out leaves open below 0, is 0
+    uni, batch = make_workload(4, seed=seed, N=2000, K=32, M=64, factor_bound=(4, 0.03), tilt=0.01, bench=True)
+    assert np.all(batch.lower >= 0) and np.all(batch.band_lo == 0)
+    res = gpu_solve(uni, batch, precision=mode)
+    assert np.all(res["status"] == prism.PRISM_CERTIFIED)
+    assert np.all(res["lambda_band"] >= -1e-12)
