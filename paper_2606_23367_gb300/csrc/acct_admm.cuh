@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
     const int slot = CL ? int(blockIdx.x) / CS : int(blockIdx.x);
     const int a = A.order ? A.order[slot] : slot;
     if (!A.active[a]) return;                       // the same answer in every CTA of the cluster
+    if constexpr (CL) cluster.sync();               // a CTA's shared memory may be written to once it has started
     const bool own = A.Cinv == nullptr, fac = GEN && A.flo != nullptr;
     // ---- shared memory behind the fixed part: C^{-1}, G, 1 / (2 d + rho) (own), the rows of B, cost rows
     const int ldc = ((K + 31) / 32) * 32 + 8;
