@@ -62,9 +62,9 @@ struct AcctShared {
     SumCount<T> turn[ACCT_WARPS];         // turnover and signed count per warp
     SumCount<T> xseg[2][ACCT_CLUSTER][SMAX];   // sector sums per CTA of the cluster
     SumCount<T> xturn[2][ACCT_CLUSTER];
-    T fmx[ACCT_WARPS][6];                 // residual maxima per warp, and per CTA of the cluster
+    T fmx[ACCT_WARPS][7];                 // residual maxima per warp, and per CTA of the cluster
     int imx[ACCT_WARPS];
-    T xmx[ACCT_CLUSTER][6];
+    T xmx[ACCT_CLUSTER][7];
     int ximx[ACCT_CLUSTER];
     T xs[SMAX];                           // where each sector is evaluated (nu, or its edge's root)
     T blo[SMAX], bhi[SMAX];
@@ -261,7 +261,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
         c1[e] = in ? A.c[base + p] : T(0);
         mu[e] = in ? A.mu[p] + (A.tilt ? A.tilt[base + p] : T(0)) : T(0);
         z[e] = (A.resume && in) ? A.z[base + p] : fmin(fmax(w0[e], lo[e]), up[e]);
-        y[e] = (A.resume && in) ? A.y[base + p] : T(0);
+        // (the tilt belongs to the costs that the projection prices, as in the batched kernels' cost rows:
+        // with y + tilt in the place of y that is the iteration with mu + tilt, started from y = tilt)
+        y[e] = !in ? T(0) : (A.resume ? A.y[base + p] : (A.tilt ? A.tilt[base + p] : T(0)));
         pw[e] = (has_pw && in) ? A.pw_idx[base + p] : -1;
         n_row += pw[e] >= 0;
         if (pw[e] >= 0) n_seg = max(n_seg, A.pw_nbp[pw[e]] - 1);
@@ -837,7 +839,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
                 rd = fmax(rd, rho * fabs(sn - so));
                 bad |= !(isfinite(xh) && isfinite(sn));
             });
-            rps = bad ? T(INFINITY) : rp;             // joins the entries' maxima below
+            rps = bad ? T(INFINITY) : rp;
             rds = bad ? T(INFINITY) : rd;
         } else {
             matvec(Ci, sh.P, [&](int k, T q) { sh.Q[k] = q; });
@@ -944,7 +946,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
         if (has_cap) theta = th;
         // ---- z, y and the residuals (the norms only where the penalty may adapt)
         const bool adapt = (it + 1) % A.adapt_every == 0;
-        T rp = rps, rd = rds, nx = T(0), nz = T(0), ny = T(0);
+        T rp = T(0), rd = T(0), nx = T(0), nz = T(0), ny = T(0);
         int flags = 0;
         unsigned codes = 0;
         if (clamped || stale) prox(clamped, nu, th);  // (else zz holds it: nu is where the last evaluation was)
@@ -958,7 +960,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
                 if (adapt) {
                     nx = fmax(nx, fabs(v[e] - y[e] * irho));
                     nz = fmax(nz, fabs(zn));
-                    ny = fmax(ny, fabs(yn));
+                    ny = fmax(ny, fabs(A.tilt ? yn - A.tilt[base + (A.plist ? A.plist[off + i0 + ib + e] : i0 + ib + e)] : yn));
                 }
                 flags |= !(isfinite(zn) && isfinite(yn));
                 // its place: inside a linear piece above or below w0, or at a breakpoint, and the same one
@@ -975,22 +977,25 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
             if (now - *A.t0 > A.budget_ns) flags |= 2;
         }
         rp = warp_maxv(rp); rd = warp_maxv(rd);
+        if (fac) { rps = warp_maxv(rps); rds = warp_maxv(rds); }
         if (adapt) { nx = warp_maxv(nx); nz = warp_maxv(nz); ny = warp_maxv(ny); }
         flags = __reduce_or_sync(0xffffffffu, unsigned(flags));
         if (lane == 0) {
             T* m = sh.fmx[warp];
             m[0] = rp; m[1] = rd;
             if (adapt) { m[2] = nx; m[3] = nz; m[4] = ny; }
+            if (fac) { m[5] = rps; m[6] = rds; }
             sh.imx[warp] = flags;
         }
         __syncthreads();
-        auto gather_max = [&](const T (*m)[6], const int* f, int count) {
+        auto gather_max = [&](const T (*m)[7], const int* f, int count) {
             const bool in = lane < count;
             rp = warp_maxv(in ? m[lane][0] : T(0)); rd = warp_maxv(in ? m[lane][1] : T(0));
             if (adapt) {
                 nx = warp_maxv(in ? m[lane][2] : T(0)); nz = warp_maxv(in ? m[lane][3] : T(0));
                 ny = warp_maxv(in ? m[lane][4] : T(0));
             }
+            if (fac) { rps = warp_maxv(in ? m[lane][5] : T(0)); rds = warp_maxv(in ? m[lane][6] : T(0)); }
             flags = __reduce_or_sync(0xffffffffu, in ? unsigned(f[lane]) : 0u);
         };
         gather_max(sh.fmx, sh.imx, NW);
@@ -998,13 +1003,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
             if (tid < CS) {
                 AcctShared<T>* o = cluster.map_shared_rank(&sh, tid);
                 T* m = o->xmx[rank];
-                m[0] = rp; m[1] = rd; m[2] = nx; m[3] = nz; m[4] = ny;
+                m[0] = rp; m[1] = rd; m[2] = nx; m[3] = nz; m[4] = ny; m[5] = rps; m[6] = rds;
                 o->ximx[rank] = flags;
             }
             cluster.sync();
             gather_max(sh.xmx, sh.ximx, CS);
         }
         ++it;
+        // the factor block's residuals take part in the stopping test; the penalty follows the entries' alone
+        const T ep = rp, ed = rd;
+        rp = fmax(rp, rps); rd = fmax(rd, rds);
         close = rp;
         // The residuals having met their target, the account goes on until its entries have kept their places
         // for A.settle iterations: the polish starts from those places
@@ -1019,8 +1027,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
         else if (it >= A.max_iter) { status = PRISM_TIMEOUT; go = false; }
         else if (flags & 2) { stopped = true; go = false; }
         else if (adapt) {
-            const T pr = rp / fmax(fmax(nx, nz), T(1e-12));
-            const T du = rd / fmax(ny, T(1e-12));
+            const T pr = ep / fmax(fmax(nx, nz), T(1e-12));
+            const T du = ed / fmax(ny, T(1e-12));
             const T ratio = sqrt(pr / fmax(du, T(1e-20)));
             int dj = int(lrint(double(RHO_PER_DECADE) * log10(double(fmax(ratio, T(1e-12))))));
             dj = max(-4, min(4, dj));

@@ -1196,12 +1196,6 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) k_polish(PolDev P, int 
                     if (sh.rows[r] == row) return sh.used[r] == 0;
                 return false;
             };
-            auto bounds_sum = [&](int s2, const double* b) {
-                double t = 0.0;
-#pragma unroll 8
-                for (int p = P.sec_start[s2]; p < P.sec_start[s2 + 1]; ++p) t += b[base + p];
-                return t;
-            };
             for (int s2 = lane; s2 < S; s2 += 32) {
                 const double ssum = sh.secsum[s2];
                 const double hi = sh.bhi_s[s2], lo = sh.blo_s[s2];
@@ -1216,11 +1210,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) k_polish(PolDev P, int 
                     if (wb > 0 ? ssum < hi : ssum > lo) { set_wb(s2, 0); ++dep_in; }
                     else ++dep_out;
                 } else if (wb == 0) {
-                    // (an edge that the bounds of the entries imply is left only because an entry left its
-                    // own bound, which the next round fixes: as a row it would leave the multiplier open,
-                    // anywhere between 0 and that of the bounds. Batched books keep either outcome)
-                    if (ssum > hi + tol_p) { ++bviol; if (!P.no_implied || bounds_sum(s2, P.up) > hi) set_wb(s2, 1); }
-                    else if (ssum < lo - tol_p) { ++bviol; if (!P.no_implied || bounds_sum(s2, P.lo) < lo) set_wb(s2, -1); }
+                    if (ssum > hi + tol_p) { ++bviol; set_wb(s2, 1); }
+                    else if (ssum < lo - tol_p) { ++bviol; set_wb(s2, -1); }
                 } else {
                     // an independent working row is off its bound only when free weights left
                     // their segments (counted in nviol): the next round solves again

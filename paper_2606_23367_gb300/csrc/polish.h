@@ -38,7 +38,6 @@ struct PolDev {
     const double* band_lo = nullptr;    // M x S
     const double* band_hi = nullptr;
     const double* tau = nullptr;        // M (+inf = none)
-    int no_implied = 0;                 // 1: a band edge that the entries' bounds imply is never a row
     const double* flo = nullptr;        // M x K factor-exposure bounds, or null (no factor rows)
     const double* fhi = nullptr;
     const int* sflag = nullptr;         // M x K: factor rows the iterations hold at a bound

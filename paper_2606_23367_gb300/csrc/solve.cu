@@ -1060,7 +1060,6 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     P.w0f = BD.w0f; P.lof = BD.lof; P.upf = BD.upf; P.cf = BD.cf;
     P.w0 = BD.w0; P.lo = BD.lo; P.up = BD.up; P.c = BD.c;
     if (!has_tilt || tilt_rows) { P.tilt = nullptr; P.tiltf = nullptr; }
-    P.no_implied = acct;
     P.pw_idx = pwidx; P.pw_bp = BD.pw_bp; P.pw_sl = BD.pw_sl; P.pw_phi_lo = (const double*)stage[6]; P.pw_nbp = BD.pw_nbp;
     P.band_lo = BD.band_lo; P.band_hi = BD.band_hi; P.tau = BD.tau;
     if (BD.has_fac) { P.flo = BD.flo; P.fhi = BD.fhi; P.sflag = D.sflag; }
