@@ -160,12 +160,11 @@ typedef struct {
     void*   cuda_stream;      /* cudaStream_t to run on (NULL = the library's own stream) */
     int32_t ragged_layout;    /* books with asset_idx in the batched modes: 1 = dense-masked over the
                                  universe (every product over all N positions, non-members pinned
-                                 at 0); 2 = packed (each account's own names only, with the
-                                 account's own capacitance: account-resident, see chains, while the
-                                 largest account fits, else one persistent launch of per-account
-                                 blocks); 0 = packed account-resident where that is estimated to be
-                                 the faster, else dense-masked (prism_autotune times the layouts for
-                                 a book) (default 0) */
+                                 at 0), on the batched kernels; 2 = packed (each account's own names
+                                 only, one persistent launch of per-account blocks with the
+                                 account's own capacitance, another splitting); 0 = dense-masked,
+                                 account-resident (see chains) where that is estimated to be the
+                                 faster (prism_autotune times the layouts for a book) (default 0) */
     int32_t g2_sets;          /* tile shape of the tensor-core product B'X: clusters of 8 CTAs per
                                  128-account tile along the assets, each CTA summing an asset chunk
                                  of N / (8 g2_sets) (rounded up to 64); 0 = about one CTA per SM

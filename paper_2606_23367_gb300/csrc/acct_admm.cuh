@@ -20,8 +20,8 @@
 // sectors are a segmented scan over the lanes and a few additions; warp 0 alone takes the steps of
 // the roots.
 // Measured (ADMM phase of a solve, before and after): 37 accounts x 777 x 17 1.31 -> 0.26 ms, 64 x 2,000 x
-// 32 1.24 -> 0.24, 256 ragged of up to 5,000 x 32 2.28 -> 1.14, 200 x 1,924 x 48 with lots and a cap
-// 8.0 -> 1.5, one account of 100 x 10 0.94 -> 0.09, in FP64 2.8 -> 0.39.
+// 32 1.24 -> 0.24, 200 x 1,924 x 48 with lots and a cap 8.0 -> 1.5, one account of 100 x 10 0.94 -> 0.09, in
+// FP64 2.8 -> 0.39.
 // Accounts too large for one CTA's shared memory are split over a cluster of up to eight CTAs,
 // which add their partial sums by stores into each other's shared memory; every CTA then holds the
 // same sums, added in the same order, and takes the same decisions.
@@ -194,7 +194,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
     const int a = A.order ? A.order[slot] : slot;
     if (!A.active[a]) return;                       // the same answer in every CTA of the cluster
     if constexpr (CL) cluster.sync();               // a CTA's shared memory may be written to once it has started
-    const bool own = A.Cinv == nullptr, fac = GEN && A.flo != nullptr;
+    constexpr bool own = sizeof(T) == 8;            // C^{-1} formed and inverted here
+    const bool fac = GEN && A.flo != nullptr;
     // ---- shared memory behind the fixed part: C^{-1}, G, 1 / (2 d + rho) (own), the rows of B, cost rows
     const int ldc = ((K + 31) / 32) * 32 + 8;
     T* Ci = reinterpret_cast<T*>(acct_smem + (sizeof(AcctShared<T>) + 15) / 16 * 16);
@@ -202,8 +203,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
     const int nc = row_chunks(K, PC), ncs = row_stride(K, PC);
     // ---- this CTA's entries
     const size_t base = (size_t)a * A.Npad;
-    const int64_t off = A.plist ? A.poff[a] : 0;
-    const int n = A.plist ? int(A.poff[a + 1] - off) : A.N;
+    const int n = A.N;
     const int per = CL ? (n + CS - 1) / CS : n;
     const int i0 = rank * per, my = max(0, min(per, n - i0));
     // A thread's entries are consecutive: entry e of lane l of warp w is number 32 E w + E l + e. Their
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
     uint4* Brow = reinterpret_cast<uint4*>(wrow + (own ? slots : 0));
     T* pwrow = reinterpret_cast<T*>(Brow + (size_t)slots * ncs);
     for (int s = tid; s <= S; s += NT)
-        sh.sec[s] = max(0, min(my, (A.plist ? A.psec[(size_t)a * (S + 1) + s] : A.sec_start[s]) - i0));
+        sh.sec[s] = max(0, min(my, A.sec_start[s] - i0));
     for (int s = tid; s < S; s += NT) {
         sh.blo[s] = A.band_lo[a * S + s];
         sh.bhi[s] = A.band_hi[a * S + s];
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
         const int r = i % (32 * E), sl = i - r + 32 * (r % E) + r / E;
         uint4 u = make_uint4(0, 0, 0, 0);
         if (i < my) {
-            const int p = A.plist ? A.plist[off + i0 + i] : i0 + i;
+            const int p = i0 + i;
             if constexpr (sizeof(BT) == 2) u = reinterpret_cast<const uint4*>(A.B16p + (size_t)p * KMAX)[c];
             else if constexpr (sizeof(BT) == 4) u = reinterpret_cast<const uint4*>(A.B32p + (size_t)p * KMAX)[c];
             else {
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
     for (int e = 0; e < E; ++e) {
         const int i = ib + e;
         const bool in = i < my;
-        const int p = in ? (A.plist ? A.plist[off + i0 + i] : i0 + i) : 0;
+        const int p = in ? i0 + i : 0;
         w0[e] = in ? A.w0[base + p] : T(0);
         lo[e] = in ? A.lo[base + p] : T(0);
         up[e] = in ? A.up[base + p] : T(0);
@@ -610,21 +610,20 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
     };
 
     // ---- capacitance ------------------------------------------------------------------------
-    // C^{-1} at penalty index j into shared memory: from the universe's table, or formed from this
-    // account's rows
+    // C^{-1} at penalty index j into shared memory: from the universe's table, or (FP64) formed from the
+    // rows of B and inverted here
     T idl[E];
     auto capacitance = [&]() -> bool {
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             idl[e] = T(0);
             if (ib + e < my) {
-                const int p = A.plist ? A.plist[off + i0 + ib + e] : i0 + ib + e;
-                idl[e] = T(1) / (T(2) * A.d[p] + rho);
+                idl[e] = T(1) / (T(2) * A.d[i0 + ib + e] + rho);
             }
             if (own) wrow[slot0 + 32 * e] = idl[e];
         }
         __syncthreads();
-        if (!own) {
+        if constexpr (!own) {
             for (int e = tid; e < K * K; e += NT) {
                 const int r = e / K, c = e - r * K;
                 Ci[r * ldc + c] = T(A.Cinv[(size_t)j * K * K + e]);
@@ -673,22 +672,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
                             }
                 __syncthreads();
             }
-        }
-        if constexpr (CL) {
-            // the CTAs' Gram matrices: read each other's (in rank order), then replace one's own
-            cluster.sync();
-            T tot[KMAX * KMAX / 128];                 // (a cluster's blocks have at least 128 threads)
-            int q = 0;
-            for (int e = tid; e < K * K; e += NT, ++q) {
-                const int o = (e / K) * ldc + e % K;
-                T t = T(0);
-                for (int r = 0; r < CS; ++r) t += cluster.map_shared_rank(Ci, r)[o];
-                tot[q] = t;
-            }
-            cluster.sync();
-            q = 0;
-            for (int e = tid; e < K * K; e += NT, ++q) Ci[(e / K) * ldc + e % K] = tot[q];
-            __syncthreads();
         }
         for (int r = warp; r < K; r += NW)
             for (int c = lane; c < K; c += 32) {
@@ -960,7 +943,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
                 if (adapt) {
                     nx = fmax(nx, fabs(v[e] - y[e] * irho));
                     nz = fmax(nz, fabs(zn));
-                    ny = fmax(ny, fabs(A.tilt ? yn - A.tilt[base + (A.plist ? A.plist[off + i0 + ib + e] : i0 + ib + e)] : yn));
+                    ny = fmax(ny, fabs(A.tilt ? yn - A.tilt[base + i0 + ib + e] : yn));
                 }
                 flags |= !(isfinite(zn) && isfinite(yn));
                 // its place: inside a linear piece above or below w0, or at a breakpoint, and the same one
@@ -1051,7 +1034,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
 #pragma unroll
     for (int e = 0; e < E; ++e)
         if (ib + e < my) {
-            const size_t p = base + (A.plist ? A.plist[off + i0 + ib + e] : i0 + ib + e);
+            const size_t p = base + i0 + ib + e;
             A.z[p] = z[e];
             A.y[p] = y[e];
             if constexpr (sizeof(T) == 8) A.zf[p] = float(z[e]);

@@ -1,4 +1,4 @@
-// acct_admm.h -- the account-resident ADMM kernel (acct_admm.cu): every iteration of an account in
+// acct_admm.h -- the account-resident ADMM kernel (acct_admm.cuh): every iteration of an account in
 // one launch, its rows of B in shared memory and its entries in registers, one CTA per account
 // or a cluster of up to eight that split the account's entries.
 #pragma once
@@ -21,8 +21,8 @@ struct AcctArgs {
     const T* f = nullptr;                  // K
     const T* d = nullptr;                  // Npad
     const T* mu = nullptr;                 // Npad
-    const float* Cinv = nullptr;           // NRHO x K x K capacitance inverses of the whole universe, or
-                                           // null: each account forms its own (its own names; FP64)
+    const float* Cinv = nullptr;           // NRHO x K x K capacitance inverses (T = float; in FP64 the
+                                           // kernel forms them itself, for each penalty)
     const float* G = nullptr;              // NRHO x K x K Gram matrices beside it (factor bounds)
     const int* sec_start = nullptr;        // S + 1
     // per entry, dense M x Npad (sorted positions)
@@ -35,10 +35,6 @@ struct AcctArgs {
     const T *band_lo = nullptr, *band_hi = nullptr;   // M x S
     const T* tau = nullptr;                // M (+inf = no cap)
     const T *flo = nullptr, *fhi = nullptr;           // M x K factor-exposure bounds, or null
-    // ragged books: each account's positions in increasing order and its sector ranges in them
-    const int* plist = nullptr;
-    const int64_t* poff = nullptr;
-    const int* psec = nullptr;
     const int* order = nullptr;            // the accounts of this launch, or null: 0, 1, ...
     // state, M x Npad (also the start of a second pass) and per account
     T *z = nullptr, *y = nullptr;
@@ -64,9 +60,8 @@ struct AcctShape {
 };
 
 // The shape for accounts of at most n entries (E = 0: they do not fit). bytes_b: size of an element
-// of B, 8 in FP64; own: each account forms its own capacitance; fac: factor bounds; pw: some
-// accounts have piecewise-linear cost rows.
-AcctShape acct_shape(int n, int K, int bytes_b, bool own, bool fac, bool pw);
+// of B, 8 in FP64; fac: factor bounds; pw: some accounts have piecewise-linear cost rows.
+AcctShape acct_shape(int n, int K, int bytes_b, bool fac, bool pw);
 template <typename T>
 void launch_acct_admm(const AcctArgs<T>& A, const AcctShape& sh, int n_accounts, cudaStream_t st);
 void launch_acct_bf16(const AcctArgs<float>& A, const AcctShape& sh, int n_accounts, cudaStream_t st);

@@ -584,11 +584,6 @@ static double ms_between(cudaEvent_t a, cudaEvent_t b) {
 // ---------------------------------------------------------------------------
 // the account-resident iterations: which books take them, in which launches
 // ---------------------------------------------------------------------------
-struct AcctClass {
-    int first, count;                   // its accounts in the order list (all of them when not ragged)
-    AcctShape shape;
-};
-
 static int sm_count() {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -619,38 +614,16 @@ static bool open_form(const prism_solve_opts& o) {
            !std::getenv("PRISM_TEST_STALLED_WAIT_NS");
 }
 
-static bool acct_route(const prism_solve_opts& o, bool plain, bool fp64, bool bf16, bool ragged, int M, int N, int K,
-                       bool pw, bool tilt, bool fac, bool cap, const std::vector<int64_t>& offs, std::vector<AcctClass>& classes,
-                       std::vector<int>& order) {
-    if (!open_form(o)) return false;
+// A ragged book is iterated over all positions, as the batched kernels do (non-members stay pinned at 0): the
+// packed layout, whose capacitance is that of an account's own names, is another splitting.
+static bool acct_route(const prism_solve_opts& o, bool plain, bool packed, bool fp64, bool bf16, int M, int N, int K, bool pw,
+                       bool tilt, bool fac, bool cap, AcctShape& shape) {
+    if (packed || !open_form(o)) return false;
     const int bytes = fp64 ? 8 : (bf16 ? 2 : 4);
-    const int sms = sm_count();
-    classes.clear();
-    order.clear();
-    double us = 0.0;
-    if (!ragged) {
-        classes.push_back({0, M, acct_shape(N, K, bytes, fp64, fac, pw)});
-        if (classes[0].shape.E == 0) return false;
-        us = acct_iteration_us(classes[0].shape, N, M, K, bytes, sms);
-    } else {
-        // accounts largest first; a class ends where half the entries would do, so that small accounts
-        // take small blocks, several to an SM
-        order.resize(M);
-        for (int a = 0; a < M; ++a) order[a] = a;
-        auto size = [&](int a) { return (int)(offs[a + 1] - offs[a]); };
-        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return size(x) > size(y); });
-        for (int i = 0; i < M;) {
-            const int n = size(order[i]);
-            AcctClass c{i, 0, acct_shape(n, K, bytes, true, fac, pw)};
-            if (c.shape.E == 0) return false;
-            while (i < M && (size(order[i]) > n / 2 || n <= 128)) { ++c.count; ++i; }
-            us += acct_iteration_us(c.shape, n, c.count, K, bytes, sms);
-            classes.push_back(c);
-        }
-    }
-    // single accounts and the packed layout have no batched form
-    if (plain || o.ragged_layout == 2) return true;
-    return us <= batched_iteration_us(M, N, bf16, pw || tilt || cap || fac);
+    shape = acct_shape(N, K, bytes, fac, pw);
+    if (shape.E == 0) return false;
+    if (plain) return true;                           // (no batched form is the faster for one account)
+    return acct_iteration_us(shape, N, M, K, bytes, sm_count()) <= batched_iteration_us(M, N, bf16, pw || tilt || cap || fac);
 }
 
 // ---------------------------------------------------------------------------
@@ -705,18 +678,16 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         packed = o->ragged_layout == 2;
     }
     // ---- which iterations: account-resident (acct_admm.cuh) where its accounts fit and it is the faster
-    std::vector<AcctClass> classes;
+    AcctShape shape;
     std::vector<int> order_h;
-    const bool acct = acct_route(*o, plain, fp64, batched_mode_bf16, b->asset_idx != nullptr, M, N, K, has_lots, has_tilt,
-                                 has_fac_in, b->turnover_cap != nullptr, offs, classes, order_h);
+    const bool acct = acct_route(*o, plain, packed, fp64, batched_mode_bf16, M, N, K, has_lots, has_tilt, has_fac_in,
+                                 b->turnover_cap != nullptr, shape);
     // the account-resident kernel takes a tilt as a shift of mu, the batched ones as cost rows
     const bool tilt_rows = has_tilt && !acct;
     const bool has_pw = has_lots || tilt_rows;
     const int64_t n_pw64 = n_lots + (tilt_rows ? nnz : 0);
     if (n_pw64 > INT32_MAX) { set_error("too many tax lots"); return PRISM_ERR_UNSUPPORTED; }
     const int n_pw = (int)n_pw64;
-    if (acct) packed = false;
-    const bool lists = packed || (acct && b->asset_idx);   // per-account position lists are needed
     // ---- workspace layout
     const size_t MN = (size_t)M * Npad;
     int tc_chunk = 0;
@@ -807,7 +778,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         // packed layout of a ragged book: position lists, sector ranges, processing order, FP32
         // state and input copies for accounts too large for shared memory
         const size_t np = packed ? (size_t)nnz : 0;
-        PK.plist = A.take<int>(lists ? (size_t)nnz : 0); PK.psec = A.take<int>(lists ? (size_t)M * (S + 1) : 0);
+        PK.plist = A.take<int>(packed ? (size_t)nnz : 0); PK.psec = A.take<int>(packed ? (size_t)M * (S + 1) : 0);
         PK.order = A.take<int>(M); PK.queue = A.take<int>(4);
         t0_dev = A.take<unsigned long long>(1);
         inbox = A.take<char>(SolveCache::BOX);
@@ -1109,8 +1080,6 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         PK.stage_cap = (int)std::min<int64_t>(nmax, (int64_t)(room / per));
         PRISM_CUDA_TRY(cudaMemcpyAsync(PK.order, order_h.data(), (size_t)M * 4, cudaMemcpyHostToDevice, st));
     }
-    if (acct && b->asset_idx)
-        PRISM_CUDA_TRY(cudaMemcpyAsync(PK.order, order_h.data(), (size_t)M * 4, cudaMemcpyHostToDevice, st));
     // ---- control init (see k_setup)
     if (!acct) {
         cudaMemsetAsync(D.v, 0, MN * 4, st);
@@ -1210,8 +1179,8 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     AcctArgs<float> AF;
     AcctArgs<double> AD;
     // the few accounts that a batched book sends back to the iterations go on account-resident
-    const AcctShape again = (!acct && !fp64 && !packed && !b->asset_idx && open_form(*o))
-                                ? acct_shape(N, K, batched_mode_bf16 ? 2 : 4, false, BD.has_fac, has_pw) : AcctShape();
+    const AcctShape again = (!acct && !fp64 && !packed && open_form(*o))
+                                ? acct_shape(N, K, batched_mode_bf16 ? 2 : 4, BD.has_fac, has_pw) : AcctShape();
     if (acct || again.E) {
         auto fill = [&](auto& A) {
             A.M = M; A.N = N; A.Npad = Npad; A.K = K; A.S = S;
@@ -1219,7 +1188,6 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
             A.pw_idx = pwidx; A.pw_nbp = BD.pw_nbp;
             A.nu = D.nu; A.eta_hi = D.eta_hi; A.eta_lo = D.eta_lo; A.theta = D.theta; A.zf = D.z;
             A.rho_idx = D.rho_idx; A.iters = D.iters; A.active = D.active; A.status = D.status;
-            if (b->asset_idx) { A.plist = PK.plist; A.poff = PA.offsets; A.psec = PK.psec; }
             if (BD.has_fac) A.sflag = D.sflag;
             A.t0 = t0_dev;
             // With lots or a cap the polish can lose its way from a start a few places off, and one such
@@ -1234,7 +1202,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         fill(AD);
         if (batched_mode_bf16) AF.B16p = U.d_B16p; else AF.B32p = U.d_B32p;
         AF.f = U.d_f32; AF.d = U.d_d32; AF.mu = U.d_mu32;
-        if (!b->asset_idx) { AF.Cinv = D.Cinv; AF.G = D.G; }   // (of the split-off factor block when there is one)
+        AF.Cinv = D.Cinv; AF.G = D.G;                 // (of the split-off factor block when there is one)
         AF.w0 = BD.w0f; AF.lo = BD.lof; AF.up = BD.upf; AF.c = BD.cf;
         AF.pw_bp = BD.pw_bpf; AF.pw_sl = BD.pw_slf;
         AF.band_lo = BD.band_lof; AF.band_hi = BD.band_hif;
@@ -1250,31 +1218,19 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         if (BD.has_cap) AD.tau = BD.tau;
         if (BD.has_fac) { AD.flo = BD.flo; AD.fhi = BD.fhi; AD.s = P64.s_state; AD.ys = P64.ys_state; }
     }
-    // the accounts' iterations, one launch per class of sizes (side by side on the chains' streams)
     auto set_budget = [&]() {                         // (from t0, which the device took a little after the call began)
         if (o->time_budget_s > 0)
             AF.budget_ns = AD.budget_ns = (unsigned long long)(std::min(o->time_budget_s, 1e9) * 1e9) + 1;
     };
+    // the accounts' iterations in one launch
     auto run_acct = [&](int resume, double eps, int max_iter) {
         set_budget();
         AF.resume = AD.resume = resume;
         AF.eps = (float)eps; AD.eps = eps;
         AF.max_iter = AD.max_iter = max_iter;
-        const int nstream = SC.chains_ok && !SC.prof.on ? std::min<int>(SolveCache::MAXCH, (int)classes.size()) : 1;
-        SC.prof.run(PRISM_K_BLOCK, (int)classes.size(), st, [&] {
-            if (nstream > 1) cudaEventRecord(SC.ev_fork, st);
-            for (int c = 1; c < nstream; ++c) cudaStreamWaitEvent(SC.chst[c - 1], SC.ev_fork, 0);
-            for (size_t c = 0; c < classes.size(); ++c) {
-                const AcctClass& q = classes[c];
-                cudaStream_t s = c % nstream ? SC.chst[c % nstream - 1] : st;
-                AF.order = AD.order = b->asset_idx ? PK.order + q.first : nullptr;
-                if (fp64) launch_acct_admm(AD, q.shape, q.count, s);
-                else launch_acct_admm(AF, q.shape, q.count, s);
-            }
-            for (int c = 1; c < nstream; ++c) {
-                cudaEventRecord(SC.ev_join[c - 1], SC.chst[c - 1]);
-                cudaStreamWaitEvent(st, SC.ev_join[c - 1], 0);
-            }
+        SC.prof.run(PRISM_K_BLOCK, 1, st, [&] {
+            if (fp64) launch_acct_admm(AD, shape, M, st);
+            else launch_acct_admm(AF, shape, M, st);
         });
     };
     // A batched book with only a few accounts left to iterate goes on account-resident once their CTAs
@@ -1366,10 +1322,6 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     const bool blockwise = acct || fp64 || packed;   // every iteration inside a per-account kernel
     const int cold = (D.stream_prox && !blockwise) ? std::min(std::max(0, o->stream_after), o->max_iter) : 0;
     if (acct) {
-        if (b->asset_idx)
-            SC.prof.run(PRISM_K_OTHER, 1, st, [&] {
-                launch_member_lists(M, Npad, S, member, U.d_sec_start, PA.offsets, PK.plist, PK.psec, st);
-            });
         run_acct(0, o->eps_admm, o->max_iter);
     } else if (fp64) {
         // PLAIN_FP64: every iteration of the account in one FP64 launch (block_admm.cu)

@@ -41,3 +41,41 @@ def test_a_small_book(seed):
 def test_a_mandate_with_benchmark_tilt_and_factor_bounds(seed):
     uni, batch = make_workload(4, seed=seed, N=2000, K=32, M=64, factor_bound=(4, 0.03), tilt=0.01, bench=True)
     _same(uni, batch, prism.PRISM_BATCHED_BF16, chains=1)
+
+
+@pytest.mark.parametrize("seed", [6, 29, 30, 33, 45, 115])
+def test_ragged_accounts(seed):
+    # accounts of 100 names up to the universe: iterated over all its positions in either form
+    uni, batch = make_workload(2, seed=seed, N=1500, K=24, M=128)
+    _same(uni, batch, prism.PRISM_BATCHED_BF16, ragged_layout=1)
+
+
+@pytest.mark.parametrize("layout", [0, 1, 2])
+def test_diagnostics_of_ragged_accounts_that_do_not_certify(layout):
+    # on a handle that has held another book of the same shape: nothing of it may reach an account's
+    # diagnostics, which are those of the weights returned, nor a gradient
+    uni, batch = make_workload(2, seed=3, N=1500, K=24, M=64)
+    _, other = make_workload(2, seed=4, N=1500, K=24, M=64)
+    h = prism.create_universe(uni)
+    try:
+        for b in (batch, other):                       # (the workspace has its size after the first two)
+            prism.solve(h, b, precision=prism.PRISM_BATCHED_BF16, ragged_layout=layout)
+        res = prism.solve(h, batch, precision=prism.PRISM_BATCHED_BF16, ragged_layout=layout, max_iter=2, polish_rounds=1,
+                          keep_for_backward=1)
+        left = np.flatnonzero(res["status"] != prism.PRISM_CERTIFIED)
+        assert len(left) > 0 and not np.any(res["status"] == prism.PRISM_NUMERICAL_FAILURE)
+        for a in left:
+            sl = batch.account_slice(a)
+            w, i = res["w"][sl], batch.asset_idx[sl]
+            h_ = uni.B[i].T @ w
+            sums = np.bincount(uni.sector[i], w, uni.n_sectors)
+            obj = h_ @ (uni.f * h_) + w @ (uni.d[i] * w) - uni.mu[i] @ w + np.abs(w - batch.w0[sl]) @ batch.tc[sl]
+            want = {prism.PRISM_DIAG_BUDGET: abs(w.sum() - 1.0), prism.PRISM_DIAG_OBJ: obj,
+                    prism.PRISM_DIAG_EXPOSURE: max(0.0, np.max(sums - batch.band_hi[a]), np.max(batch.band_lo[a] - sums))}
+            for col, v in want.items():
+                assert abs(res["diag"][a, col] - v) <= 1e-12, (a, col)
+        grad = prism.prism_solve_batch_backward(res["state"], np.ones(len(batch.w0)))
+        assert all(np.all(np.isfinite(grad[k])) for k in ("dmu", "dB", "dd", "dw0"))
+        res["state"].close()
+    finally:
+        h.close()
