@@ -591,20 +591,24 @@ static int sm_count() {
     return std::max(1, sms);
 }
 
-// Time of one iteration of the whole book, us, as measured at 500 to 10,000 assets, 16 to 64 factors and
-// 16 to 500 accounts. Account-resident: 4.5 for the chain of reductions, 2.5 more when it crosses a
-// cluster, and the products with the CTA's rows; times the waves of clusters.
-static double acct_iteration_us(const AcctShape& s, int n, int M, int K, int bytes, int sms) {
+// Time of one iteration of the whole book, us, fitted to both routes' times over 741 books (300 to 10,000
+// assets, 10 to 64 factors, 2 to 400 accounts; the L1 cost in BF16 and FP32, and in BF16 lots, tilts, caps,
+// factor bounds and ragged accounts). Account-resident: 4.5 for the chain of reductions, 2.5 more when it
+// crosses a cluster, and the products with the CTA's rows; times the book's share of the SMs.
+// Batched: the latency of the launches (with the iterations that a chunk runs past the last account's)
+// and the traffic; lots and tilts are priced by rows, a cap by repeated budget roots. Of the 741
+// choices 8 take longer than the other route by 10 to 24% (400 ragged x 3,000 x 16 the most: batched 1.96
+// against 1.57 ms of iterations). Lots keep the line that they had: two books of 2 million entries would be
+// 2.2 and 2.6 times as fast account-resident.
+static double acct_iteration_us(const AcctShape& s, int n, int M, int K, int sms) {
     const int regs = s.threads > 256 ? 128 : 232;
     const int per_sm = std::max(1, std::min((int)(228 * 1024 / (s.smem + 1024)), 65536 / (s.threads * regs)));
-    const double at_once = std::max(1.0, (s.cluster > 4 ? 0.85 : 1.0) * sms * per_sm / s.cluster);
-    const double one = 4.5 + (s.cluster > 1 ? 2.5 : 0.0) + (bytes > 2 ? 6e-5 : 5e-5) * cdiv(n, s.cluster) * K;
-    return std::ceil(M / at_once) * one * (per_sm > 1 ? 1.3 : 1.0);
+    const double waves = std::max(1.0, double(M) * s.cluster / (double(sms) * per_sm));
+    return waves * (4.5 + (s.cluster > 1 ? 2.5 : 0.0) + 4e-5 * cdiv(n, s.cluster) * K) * (per_sm > 1 ? 1.3 : 1.0);
 }
-// Batched: the latency of its launches (with the iterations that a chunk runs past the last account's)
-// and the traffic; books with tax lots, tilts, caps or factor bounds take the staged prox on every call.
-static double batched_iteration_us(int M, int N, bool bf16, bool staged) {
-    return (staged ? 60.0 : 30.0) + (bf16 ? 9e-6 : 3e-5) * M * N;
+static double batched_iteration_us(int M, int N, bool bf16, bool lots, bool tilt, bool cap) {
+    if (lots || tilt) return 60.0 + (lots ? 9e-6 : 5e-5) * M * N;
+    return bf16 && !cap ? 33.0 + 7e-6 * M * N : 40.0 + 3e-5 * M * N;
 }
 
 // Whether the options leave the form of the iterations open: one that names a form of the batched
@@ -623,7 +627,7 @@ static bool acct_route(const prism_solve_opts& o, bool plain, bool packed, bool 
     shape = acct_shape(N, K, bytes, fac, pw);
     if (shape.E == 0) return false;
     if (plain) return true;                           // (no batched form is the faster for one account)
-    return acct_iteration_us(shape, N, M, K, bytes, sm_count()) <= batched_iteration_us(M, N, bf16, pw || tilt || cap || fac);
+    return acct_iteration_us(shape, N, M, K, sm_count()) <= batched_iteration_us(M, N, bf16, pw, tilt, cap);
 }
 
 // ---------------------------------------------------------------------------
@@ -680,8 +684,12 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     // ---- which iterations: account-resident (acct_admm.cuh) where its accounts fit and it is the faster
     AcctShape shape;
     std::vector<int> order_h;
-    const bool acct = acct_route(*o, plain, packed, fp64, batched_mode_bf16, M, N, K, has_lots, has_tilt, has_fac_in,
-                                 b->turnover_cap != nullptr, shape);
+    auto route = [&](bool cap) {
+        return acct_route(*o, plain, packed, fp64, batched_mode_bf16, M, N, K, has_lots, has_tilt, has_fac_in, cap, shape);
+    };
+    // (whether some cap is finite is known once the device has looked at them, see below; until then only
+    // the layout of a tilt depends on the route, and with a tilt the caps do not change it)
+    bool acct = route(false);
     // the account-resident kernel takes a tilt as a shift of mu, the batched ones as cost rows
     const bool tilt_rows = has_tilt && !acct;
     const bool has_pw = has_lots || tilt_rows;
@@ -960,6 +968,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         PRISM_CUDA_TRY(cudaStreamSynchronize(st));
         const int herr = flags[0];
         BD.has_cap = flags[2] != 0;
+        acct = route(BD.has_cap);
         if (!has_lots && !flags[1]) pwidx = nullptr;      // every tilt is zero: plain costs throughout
         struct { int bit, code; const char* text; } lot_errors[] = {
             {ERR_LOT_OFFSETS, PRISM_ERR_ARGUMENT, "lot_offsets must be nondecreasing"},
