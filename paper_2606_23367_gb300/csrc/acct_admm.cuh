@@ -172,7 +172,7 @@ struct ARoot {
 };
 
 __device__ __forceinline__ float acct_rho(float, int j) { return float(RHO_MIN) * exp10f(float(j) / float(RHO_PER_DECADE)); }
-__device__ __forceinline__ double acct_rho(double, int j) { return RHO_MIN * exp10(double(j) / double(RHO_PER_DECADE)); }
+__device__ __forceinline__ double acct_rho(double, int) { return 0.0; }    // (FP64 penalties are on no grid)
 
 __device__ __forceinline__ float warp_maxv(float v) {      // of values >= 0 (a NaN is reported apart)
     return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
@@ -327,8 +327,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
         }
     }
     int j = A.rho_idx[a];
-    T rho = acct_rho(T(0), j), irho = T(1) / rho;
-    T nu = T(A.nu[a]), theta = GEN ? T(A.theta[a]) : T(0);
+    T rho = own ? (A.resume ? A.rho_state[a] : A.rho0) : acct_rho(T(0), j), irho = T(1) / rho;
+    T nu = T(A.nu[a]), theta = T(0);
+    if (GEN) theta = own ? (A.resume ? A.theta_state[a] : T(0)) : T(A.theta[a]);
     int it = A.iters[a];
     const T tau = (GEN && A.tau) ? A.tau[a] : T(INFINITY);
     const bool has_cap = GEN && isfinite(tau);
@@ -610,8 +611,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
     };
 
     // ---- capacitance ------------------------------------------------------------------------
-    // C^{-1} at penalty index j into shared memory: from the universe's table, or (FP64) formed from the
-    // rows of B and inverted here
+    // C^{-1} at the penalty into shared memory: from the universe's table (index j), or (FP64) formed from
+    // the rows of B and inverted here
     T idl[E];
     auto capacitance = [&]() -> bool {
 #pragma unroll
@@ -1005,11 +1006,20 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
         if (!met && it >= A.min_iter && rp <= A.eps && rd <= A.eps) met = it;
         // ---- control, the same in every thread
         int newj = j;
+        T newrho = rho;
         if (flags & 1) { status = PRISM_NUMERICAL_FAILURE; go = false; }
         else if (met && (quiet >= A.settle || it - met >= A.settle_max)) go = false;
         else if (it >= A.max_iter) { status = PRISM_TIMEOUT; go = false; }
         else if (flags & 2) { stopped = true; go = false; }
-        else if (adapt) {
+        else if (adapt && own) {
+            // FP64 (as in block_admm.cu): any penalty, followed by all residuals, once they are a factor of
+            // four apart
+            const T tiny = T(1e-35);
+            const T pr = rp / fmax(fmax(nx, nz), tiny), du = rd / fmax(ny, tiny);
+            const T ratio = sqrt(pr / fmax(du, tiny));
+            if (ratio > T(2) || ratio < T(0.5)) newrho = rho * fmin(fmax(ratio, T(0.1)), T(10));
+            newrho = fmin(fmax(newrho, T(1e-6)), T(1e6));
+        } else if (adapt) {
             const T pr = ep / fmax(fmax(nx, nz), T(1e-12));
             const T du = ed / fmax(ny, T(1e-12));
             const T ratio = sqrt(pr / fmax(du, T(1e-20)));
@@ -1023,9 +1033,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
             if (x > nu) sh.wh[tid] = x;
             if (x < nu) sh.wl[tid] = x;
         }
-        if (newj != j) {
+        if (newj != j || newrho != rho) {
             j = newj;
-            rho = acct_rho(T(0), j);
+            rho = own ? newrho : acct_rho(T(0), j);
             irho = T(1) / rho;
             fresh = true;
         }
@@ -1057,6 +1067,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
             A.nu[a] = float(nu);
             A.theta[a] = float(theta);
             A.rho_idx[a] = j;
+            if constexpr (own) {
+                A.rho_state[a] = rho;
+                A.theta_state[a] = theta;
+            }
             A.iters[a] = it;
             if (status) A.status[a] = status;
             if (!stopped) A.active[a] = 0;

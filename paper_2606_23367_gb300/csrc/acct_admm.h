@@ -42,6 +42,8 @@ struct AcctArgs {
     float *nu = nullptr, *eta_hi = nullptr, *eta_lo = nullptr, *theta = nullptr;
     int *rho_idx = nullptr, *iters = nullptr, *active = nullptr, *status = nullptr, *sflag = nullptr;
     T *s = nullptr, *ys = nullptr;         // M x K (factor-exposure block)
+    T *rho_state = nullptr, *theta_state = nullptr;   // FP64: the penalty and the cap's multiplier (M)
+    T rho0 = T(3);                         // FP64: the first penalty
     const unsigned long long* t0 = nullptr;   // device clock at the start of the solve
     unsigned long long budget_ns = 0;      // time budget from t0 (0: none)
     T alpha = T(1.5), eps = T(5e-4);

@@ -1224,6 +1224,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         AD.pw_bp = BD.pw_bp; AD.pw_sl = BD.pw_sl;
         AD.band_lo = BD.band_lo; AD.band_hi = BD.band_hi;
         AD.z = P64.z; AD.y = P64.y;
+        AD.rho_state = P64.rho_state; AD.theta_state = P64.theta_state; AD.rho0 = o->rho0;
         if (BD.has_cap) AD.tau = BD.tau;
         if (BD.has_fac) { AD.flo = BD.flo; AD.fhi = BD.fhi; AD.s = P64.s_state; AD.ys = P64.ys_state; }
     }

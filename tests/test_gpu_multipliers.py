@@ -79,3 +79,16 @@ def test_diagnostics_of_ragged_accounts_that_do_not_certify(layout):
         res["state"].close()
     finally:
         h.close()
+
+
+@pytest.mark.parametrize("seed", [13, 0])
+def test_fp64_iterations_are_those_of_the_blocks(seed):
+    # the same penalties in FP64, so the same iterates up to rounding: they stop at the same iteration, or at the
+    # next where a residual sits on the target
+    uni, batch = make_workload(1, seed=seed, N=777, K=17, M=37)
+    new = gpu_solve(uni, batch, precision=prism.PRISM_PLAIN_FP64)
+    old = gpu_solve(uni, batch, precision=prism.PRISM_PLAIN_FP64, chains=1)
+    assert np.array_equal(new["status"], old["status"]) and np.all(old["status"] == prism.PRISM_CERTIFIED)
+    assert int(np.max(np.abs(new["iters"] - old["iters"]))) <= 1
+    for k in ("w", "nu", "lambda_band"):
+        assert float(np.max(np.abs(new[k] - old[k]))) <= 1e-11, k
