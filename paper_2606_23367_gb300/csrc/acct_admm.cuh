@@ -765,94 +765,97 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
     bool go = true, fresh = true;                     // fresh: a new penalty
     int status = 0;
     bool stopped = false;                             // out of time, still iterating
+    bool closing = false;                             // stopped: the last iterate's root is taken to its tolerance
     bool watch = false;                               // near the target: the entries' places are followed
     unsigned held = 0;                                // this thread's entries' places, two bits each
     int quiet = 0, met = 0;                           // iterations without a change; where the target was met
     int pbuf = 0;
     while (go) {
-        if (fresh) {
-            if (!capacitance()) { status = PRISM_NUMERICAL_FAILURE; break; }
-            fresh = false;
-        }
-        // ---- X and P = B'X
-#pragma unroll
-        for (int e = 0; e < E; ++e) X[e] = (mu[e] + rho * z[e] - y[e]) * idl[e];
-        for (int h = 0; h < K; h += 32) {
-            if (K - h > 16) products(h, std::integral_constant<int, 32>());
-            else products(h, std::integral_constant<int, 16>());
-        }
-        __syncthreads();
-        if constexpr (CL) {
-            if (tid < K) {
-                T t = T(0);
-                for (int w = 0; w < NW; ++w) t += sh.part[w][tid];
-                for (int r = 0; r < CS; ++r) cluster.map_shared_rank(&sh, r)->xp[pbuf][rank][tid] = t;
-            }
-            cluster.sync();
-            if (tid < K) {
-                T t = T(0);
-                for (int r = 0; r < CS; ++r) t += sh.xp[pbuf][r][tid];
-                sh.P[tid] = t;
-            }
-            pbuf ^= 1;
-        } else if (tid < K) {
-            T t0 = T(0), t1 = T(0);
-            int w = 0;
-            for (; w + 1 < NW; w += 2) { t0 += sh.part[w][tid]; t1 += sh.part[w + 1][tid]; }
-            if (w < NW) t0 += sh.part[w][tid];
-            sh.P[tid] = t0 + t1;
-        }
-        __syncthreads();
-        // ---- Q = C^{-1} P; with the factor block (s = B'x, dual ys) Q' = C^{-1}(P + G tv) - tv,
-        // tv = rho s - ys, and B'x = P - G Q'
         T rps = T(0), rds = T(0);
-        if (fac) {
-            if (tid < K) { sh.tv[tid] = rho * sh.s[tid] - sh.ys[tid]; sh.P0[tid] = sh.P[tid]; }
+        if (!closing) {
+            if (fresh) {
+                if (!capacitance()) { status = PRISM_NUMERICAL_FAILURE; break; }
+                fresh = false;
+            }
+            // ---- X and P = B'X
+#pragma unroll
+            for (int e = 0; e < E; ++e) X[e] = (mu[e] + rho * z[e] - y[e]) * idl[e];
+            for (int h = 0; h < K; h += 32) {
+                if (K - h > 16) products(h, std::integral_constant<int, 32>());
+                else products(h, std::integral_constant<int, 16>());
+            }
             __syncthreads();
-            matvec(Gm, sh.tv, [&](int k, T g) { sh.P[k] = sh.P0[k] + g; });
-            matvec(Ci, sh.P, [&](int k, T q) { sh.Q[k] = q - sh.tv[k]; });
-            T rp = T(0), rd = T(0);
-            int bad = 0;
-            matvec(Gm, sh.Q, [&](int k, T g) {
-                const T bx = sh.P0[k] - g, so = sh.s[k], yo = sh.ys[k];
-                const T xh = A.alpha * bx + (T(1) - A.alpha) * so;
-                const T sn = fmin(fmax(xh + yo * irho, A.flo[(size_t)a * K + k]), A.fhi[(size_t)a * K + k]);
-                sh.s[k] = sn;
-                sh.ys[k] = yo + rho * (xh - sn);
-                rp = fmax(rp, fabs(xh - sn));
-                rd = fmax(rd, rho * fabs(sn - so));
-                bad |= !(isfinite(xh) && isfinite(sn));
-            });
-            rps = bad ? T(INFINITY) : rp;
-            rds = bad ? T(INFINITY) : rd;
-        } else {
-            matvec(Ci, sh.P, [&](int k, T q) { sh.Q[k] = q; });
-        }
-        // ---- B Q, x and v
-        T bq[E];
-        {
-            T2 acc[E];
-#pragma unroll
-            for (int e = 0; e < E; ++e) acc[e].x = acc[e].y = T(0);
-#pragma unroll 2
-            for (int c = 0; c < nc; ++c) {
-                T2 q2[PC / 2];
-#pragma unroll
-                for (int q = 0; q < PC / 2; ++q) q2[q] = reinterpret_cast<const T2*>(sh.Q)[c * (PC / 2) + q];
-#pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    const Ch b(Brow[(slot0 + 32 * e) * ncs + c]);
-#pragma unroll
-                    for (int q = 0; q < PC / 2; ++q) fma2(acc[e], b.v[q], q2[q]);
+            if constexpr (CL) {
+                if (tid < K) {
+                    T t = T(0);
+                    for (int w = 0; w < NW; ++w) t += sh.part[w][tid];
+                    for (int r = 0; r < CS; ++r) cluster.map_shared_rank(&sh, r)->xp[pbuf][rank][tid] = t;
                 }
+                cluster.sync();
+                if (tid < K) {
+                    T t = T(0);
+                    for (int r = 0; r < CS; ++r) t += sh.xp[pbuf][r][tid];
+                    sh.P[tid] = t;
+                }
+                pbuf ^= 1;
+            } else if (tid < K) {
+                T t0 = T(0), t1 = T(0);
+                int w = 0;
+                for (; w + 1 < NW; w += 2) { t0 += sh.part[w][tid]; t1 += sh.part[w + 1][tid]; }
+                if (w < NW) t0 += sh.part[w][tid];
+                sh.P[tid] = t0 + t1;
+            }
+            __syncthreads();
+            // ---- Q = C^{-1} P; with the factor block (s = B'x, dual ys) Q' = C^{-1}(P + G tv) - tv,
+            // tv = rho s - ys, and B'x = P - G Q'
+            if (fac) {
+                if (tid < K) { sh.tv[tid] = rho * sh.s[tid] - sh.ys[tid]; sh.P0[tid] = sh.P[tid]; }
+                __syncthreads();
+                matvec(Gm, sh.tv, [&](int k, T g) { sh.P[k] = sh.P0[k] + g; });
+                matvec(Ci, sh.P, [&](int k, T q) { sh.Q[k] = q - sh.tv[k]; });
+                T rp = T(0), rd = T(0);
+                int bad = 0;
+                matvec(Gm, sh.Q, [&](int k, T g) {
+                    const T bx = sh.P0[k] - g, so = sh.s[k], yo = sh.ys[k];
+                    const T xh = A.alpha * bx + (T(1) - A.alpha) * so;
+                    const T sn = fmin(fmax(xh + yo * irho, A.flo[(size_t)a * K + k]), A.fhi[(size_t)a * K + k]);
+                    sh.s[k] = sn;
+                    sh.ys[k] = yo + rho * (xh - sn);
+                    rp = fmax(rp, fabs(xh - sn));
+                    rd = fmax(rd, rho * fabs(sn - so));
+                    bad |= !(isfinite(xh) && isfinite(sn));
+                });
+                rps = bad ? T(INFINITY) : rp;
+                rds = bad ? T(INFINITY) : rd;
+            } else {
+                matvec(Ci, sh.P, [&](int k, T q) { sh.Q[k] = q; });
+            }
+            // ---- B Q, x and v
+            T bq[E];
+            {
+                T2 acc[E];
+#pragma unroll
+                for (int e = 0; e < E; ++e) acc[e].x = acc[e].y = T(0);
+#pragma unroll 2
+                for (int c = 0; c < nc; ++c) {
+                    T2 q2[PC / 2];
+#pragma unroll
+                    for (int q = 0; q < PC / 2; ++q) q2[q] = reinterpret_cast<const T2*>(sh.Q)[c * (PC / 2) + q];
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const Ch b(Brow[(slot0 + 32 * e) * ncs + c]);
+#pragma unroll
+                        for (int q = 0; q < PC / 2; ++q) fma2(acc[e], b.v[q], q2[q]);
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < E; ++e) bq[e] = acc[e].x + acc[e].y;
             }
 #pragma unroll
-            for (int e = 0; e < E; ++e) bq[e] = acc[e].x + acc[e].y;
-        }
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const T x = X[e] - bq[e] * idl[e];
-            v[e] = A.alpha * x + (T(1) - A.alpha) * z[e] + y[e] * irho;
+            for (int e = 0; e < E; ++e) {
+                const T x = X[e] - bq[e] * idl[e];
+                v[e] = A.alpha * x + (T(1) - A.alpha) * z[e] + y[e] * irho;
+            }
         }
         // ---- the projection's multipliers
         T th = T(0);
@@ -934,6 +937,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
         int flags = 0;
         unsigned codes = 0;
         if (clamped || stale) prox(clamped, nu, th);  // (else zz holds it: nu is where the last evaluation was)
+        if (closing) {
+#pragma unroll
+            for (int e = 0; e < E; ++e) { z[e] = zz[e]; y[e] = rho * (v[e] - zz[e]); }
+            break;
+        }
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const T zn = zz[e];
@@ -1027,6 +1035,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
             dj = max(-4, min(4, dj));
             newj = max(0, min(NRHO - 1, j + dj));
         }
+        // a point whose budget sum nobody looked at (stale) is closed once: an account that does not certify
+        // is returned as it stops
+        if (!go && stale && !(flags & 1)) { go = closing = true; close = T(0); }
         if (tid < S && clamped) {
             // warm starts of the edges
             const T x = sh.xs[tid];
