@@ -1017,8 +1017,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
         T newrho = rho;
         if (flags & 1) { status = PRISM_NUMERICAL_FAILURE; go = false; }
         else if (met && (quiet >= A.settle || it - met >= A.settle_max)) go = false;
-        else if (it >= A.max_iter) { status = PRISM_TIMEOUT; go = false; }
-        else if (flags & 2) { stopped = true; go = false; }
+        else if (it >= A.max_iter || (flags & 2)) {
+            // (past the target it only waited for its entries to settle)
+            if (!met && it >= A.max_iter) status = PRISM_TIMEOUT;
+            else stopped = !met;
+            go = false;
+        }
         else if (adapt && own) {
             // FP64 (as in block_admm.cu): any penalty, followed by all residuals, once they are a factor of
             // four apart

@@ -1,5 +1,7 @@
 """How accounts of the account-resident iterations stop: the point they stop at, the status they get, and
 what a time budget does."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -29,3 +31,20 @@ def test_the_point_an_account_stops_at_meets_its_budget(mode, N, K, tol, max_ite
     assert left.any()
     rounding = 32 * 2.0**-24 if mode != prism.PRISM_PLAIN_FP64 else 2.0**-24
     assert float(np.max(res["diag"][left, prism.PRISM_DIAG_BUDGET])) <= tol + rounding
+
+
+def test_an_account_that_met_its_target_is_not_timed_out():
+    # under a cap an account goes on past its target until its entries settle: the iteration cap ends that wait
+    # and is no timeout. With 60 sectors more bands bind than the polish takes rows (22) for one account, so
+    # that its status comes from the iterations; min_iter puts the target's iteration (40) below the cap (45)
+    uni, batch = make_workload(1, N=900, K=24, S=60, M=4, band_hi=0.03)
+    r = np.random.default_rng(3)
+    lower = np.where((batch.upper > 0.002) & (r.random(batch.lower.shape) < 0.05), 0.001, 0.0)
+    band_lo = np.zeros_like(batch.band_lo)
+    band_lo[:, ::7] = 0.012
+    batch = dataclasses.replace(batch, tc=r.uniform(5e-4, 5e-3, size=batch.tc.shape), lower=lower, band_lo=band_lo,
+                                turnover_cap=np.full(4, 5.0))
+    opts = dict(precision=prism.PRISM_BATCHED_BF16, min_iter=40, max_iter=15, eps_admm=0.1, eps_kkt=1e-4)
+    new, old = gpu_solve(uni, batch, **opts), gpu_solve(uni, batch, chains=1, **opts)
+    assert old["status"].tolist().count(prism.PRISM_FEASIBLE_NONCERTIFIED) == 1
+    assert np.array_equal(new["status"], old["status"])
