@@ -130,7 +130,8 @@ typedef struct {
     double  rho0;             /* initial ADMM penalty (default 3.0) */
     double  alpha;            /* over-relaxation (default 1.5) */
     double  time_budget_s;    /* wall-clock ceiling for the call (<= 0: none); looked at after every
-                                 captured chunk of iterations, account-resident after every iteration */
+                                 captured chunk of iterations, account-resident after every
+                                 iteration (PRISM_PLAIN_FP64: see there) */
     int32_t max_iter;         /* ADMM iteration cap per account (default 4000) */
     int32_t check_every;      /* iterations per captured graph launch (default 20) */
     int32_t min_iter;         /* iterations before a convergence test may stop an account */

@@ -1229,8 +1229,8 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         if (BD.has_fac) { AD.flo = BD.flo; AD.fhi = BD.fhi; AD.s = P64.s_state; AD.ys = P64.ys_state; }
     }
     auto set_budget = [&]() {                         // (from t0, which the device took a little after the call began)
-        if (o->time_budget_s > 0)
-            AF.budget_ns = AD.budget_ns = (unsigned long long)(std::min(o->time_budget_s, 1e9) * 1e9) + 1;
+        if (o->time_budget_s > 0)                     // (FP64 iterations run through: checked between accounts)
+            AF.budget_ns = (unsigned long long)(std::min(o->time_budget_s, 1e9) * 1e9) + 1;
     };
     // the accounts' iterations in one launch
     auto run_acct = [&](int resume, double eps, int max_iter) {

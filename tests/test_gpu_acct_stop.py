@@ -48,3 +48,11 @@ def test_an_account_that_met_its_target_is_not_timed_out():
     new, old = gpu_solve(uni, batch, **opts), gpu_solve(uni, batch, chains=1, **opts)
     assert old["status"].tolist().count(prism.PRISM_FEASIBLE_NONCERTIFIED) == 1
     assert np.array_equal(new["status"], old["status"])
+
+
+def test_fp64_accounts_run_through_a_time_budget():
+    # PLAIN_FP64 looks at the budget between accounts, not within one
+    uni, batch = make_workload(1, N=300, K=10, M=4)
+    res = [gpu_solve(uni, batch, precision=prism.PRISM_PLAIN_FP64, time_budget_s=t) for t in (0.0, 1e-9)]
+    assert np.array_equal(res[0]["iters"], res[1]["iters"]) and np.array_equal(res[0]["w"], res[1]["w"])
+    assert np.all(res[1]["status"] == prism.PRISM_CERTIFIED)
