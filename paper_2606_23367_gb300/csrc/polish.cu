@@ -1074,7 +1074,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) k_polish(PolDev P, int 
         const int ntiles = cdiv(N, 32);
         // the per-entry inputs of a tile; the next tile's are loaded before the current one
         // is processed, so that their latency overlaps its product and checks
-        struct TileIn { int code, pw, sec; float w0, lo, up, c, mu, bn1; };
+        struct TileIn { int code, pw, sec; float w0, lo, up, c, mu, amu, bn1; };
         auto load_tile = [&](int ti, TileIn& t) {
             const int p = ti * 32 + lane;
             const size_t e = base + p;
@@ -1082,7 +1082,9 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) k_polish(PolDev P, int 
             t.pw = P.pw_idx ? P.pw_idx[e] : -1;
             t.sec = P.sector[p];
             t.w0 = P.w0f[e]; t.lo = P.lof[e]; t.up = P.upf[e]; t.c = P.cf[e];
-            t.mu = P.tiltf ? P.mu32[p] + P.tiltf[e] : P.mu32[p];
+            const float m = P.mu32[p], tl = P.tiltf ? P.tiltf[e] : 0.f;
+            t.mu = m + tl;
+            t.amu = fabsf(m) + fabsf(tl);                 // (the two may cancel: their rounding does not)
             t.bn1 = P.Bn1f[p];
         };
         TileIn cur{}, nxt{};
@@ -1092,7 +1094,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) k_polish(PolDev P, int 
             const int p = ti * 32 + lane;                 // entries of padding (p >= N) are skipped below
             const int code = cur.code, pwv = cur.pw, sec = cur.sec;
             const float w0v = cur.w0, lov = cur.lo, upv = cur.up, cv = cur.c;
-            const float muf = cur.mu, bn1f = cur.bn1;
+            const float muf = cur.mu, amu = cur.amu, bn1f = cur.bn1;
             // g32 = B_p . fh for the tile's 32 rows: four rows of 64 floats per group of 8 lanes x 4
             // float4, coalesced over the tile's contiguous 8 KB; lane p ends with its own row
             float g32 = 0.f;
@@ -1135,7 +1137,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) k_polish(PolDev P, int 
                 const float right = (w0v > 0.f) ? -(cv + theta_f) : cv + theta_f;
                 const float up = -rr - right;
                 const float delta =
-                    1e-5f * (2.f * bn1f * fhmax_f + fabsf(muf) + fabsf(nu_f) + fabsf(lam_f) + cv + theta_f) + 1e-9f;
+                    1e-5f * (2.f * bn1f * fhmax_f + amu + fabsf(nu_f) + fabsf(lam_f) + cv + theta_f) + 1e-9f;
                 if (up < -delta) {
                     if (-up < fmargin) { fmargin = -up; fwho = p + 1; }
                     need = false;

@@ -56,3 +56,19 @@ def test_fp64_accounts_run_through_a_time_budget():
     res = [gpu_solve(uni, batch, precision=prism.PRISM_PLAIN_FP64, time_budget_s=t) for t in (0.0, 1e-9)]
     assert np.array_equal(res[0]["iters"], res[1]["iters"]) and np.array_equal(res[0]["w"], res[1]["w"])
     assert np.all(res[1]["status"] == prism.PRISM_CERTIFIED)
+
+
+@pytest.mark.parametrize("shift", [64.0, 1024.0, 8192.0])
+def test_a_tilt_that_cancels_mu_is_certified_on_exact_conditions(shift):
+    # mu + shift and a tilt of -shift: the same problem, whose FP32 sum is off by the rounding of the large
+    # terms. A certified account has the weights of the book without the shift (FP64 rounds mu + shift to
+    # 2^-53 x 8192 = 9e-13, at a curvature of 0.01 or more)
+    uni, batch = make_workload(4, N=900, K=16, M=16)
+    base = gpu_solve(uni, batch, precision=prism.PRISM_BATCHED_BF16)
+    assert np.all(base["status"] == prism.PRISM_CERTIFIED)
+    uni2 = dataclasses.replace(uni, mu=uni.mu + shift)
+    res = gpu_solve(uni2, dataclasses.replace(batch, mu_tilt=np.full(len(batch.w0), -shift)),
+                    precision=prism.PRISM_BATCHED_BF16, max_iter=30, polish_rounds=60)
+    assert np.mean(res["status"] == prism.PRISM_CERTIFIED) >= 0.5
+    sure = np.repeat(res["status"] == prism.PRISM_CERTIFIED, np.diff(batch.offsets))
+    assert float(np.max(np.abs(res["w"] - base["w"])[sure])) <= 1e-9
