@@ -1095,11 +1095,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_acct_admm(AcctArgs<T> A) {
 }
 
 template <typename T, typename BT, int E, int THREADS, bool GEN, bool CL>
-static void launch_one(const AcctArgs<T>& A0, const AcctShape& sh, int n_accounts, cudaStream_t st) {
+static cudaError_t launch_one(const AcctArgs<T>& A0, const AcctShape& sh, int n_accounts, cudaStream_t st) {
     AcctArgs<T> A = A0;
     A.pw_rows = sh.pw_rows;
     auto* k = k_acct_admm<T, BT, E, THREADS, GEN, CL>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
+    // (the limit belongs to the process: every thread sets the same one, whatever it launches with)
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ACCT_SMEM);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)n_accounts * sh.cluster);
     cfg.blockDim = dim3(sh.threads);
@@ -1111,27 +1113,25 @@ static void launch_one(const AcctArgs<T>& A0, const AcctShape& sh, int n_account
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = CL ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, k, A);
+    return cudaLaunchKernelEx(&cfg, k, A);
 }
 
 // The shapes that acct_shape gives.
 template <typename BT, bool GEN>
-static void launch_acct_gen(const AcctArgs<float>& A, const AcctShape& sh, int n, cudaStream_t st) {
+static cudaError_t launch_acct_gen(const AcctArgs<float>& A, const AcctShape& sh, int n, cudaStream_t st) {
     const bool small = sh.threads <= 256;             // (with twice the registers a thread)
     if (sh.cluster > 1) {
-        if (small) launch_one<float, BT, 4, 256, GEN, true>(A, sh, n, st);
-        else launch_one<float, BT, 4, 512, GEN, true>(A, sh, n, st);
-    } else if (sh.E == 1) {
-        launch_one<float, BT, 1, 256, GEN, false>(A, sh, n, st);
-    } else {
-        if (small) launch_one<float, BT, 4, 256, GEN, false>(A, sh, n, st);
-        else launch_one<float, BT, 4, 512, GEN, false>(A, sh, n, st);
+        if (small) return launch_one<float, BT, 4, 256, GEN, true>(A, sh, n, st);
+        return launch_one<float, BT, 4, 512, GEN, true>(A, sh, n, st);
     }
+    if (sh.E == 1) return launch_one<float, BT, 1, 256, GEN, false>(A, sh, n, st);
+    if (small) return launch_one<float, BT, 4, 256, GEN, false>(A, sh, n, st);
+    return launch_one<float, BT, 4, 512, GEN, false>(A, sh, n, st);
 }
 template <typename BT>
-static void launch_acct_float(const AcctArgs<float>& A, const AcctShape& sh, int n, cudaStream_t st) {
-    if (A.pw_idx || A.flo || A.tau) launch_acct_gen<BT, true>(A, sh, n, st);
-    else launch_acct_gen<BT, false>(A, sh, n, st);
+static cudaError_t launch_acct_float(const AcctArgs<float>& A, const AcctShape& sh, int n, cudaStream_t st) {
+    if (A.pw_idx || A.flo || A.tau) return launch_acct_gen<BT, true>(A, sh, n, st);
+    return launch_acct_gen<BT, false>(A, sh, n, st);
 }
 
 }  // namespace prism

@@ -9,6 +9,7 @@ namespace prism {
 
 constexpr int ACCT_THREADS = 512;       // largest block
 constexpr int ACCT_CLUSTER = 8;         // largest cluster
+constexpr size_t ACCT_SMEM = 227 * 1024;   // shared memory of a CTA at most
 
 // T: the arithmetic; the rows of B are kept as BF16 (bf16 mode), FP32 or FP64 (T = double)
 template <typename T>
@@ -65,8 +66,8 @@ struct AcctShape {
 // of B, 8 in FP64; fac: factor bounds; pw: some accounts have piecewise-linear cost rows.
 AcctShape acct_shape(int n, int K, int bytes_b, bool fac, bool pw);
 template <typename T>
-void launch_acct_admm(const AcctArgs<T>& A, const AcctShape& sh, int n_accounts, cudaStream_t st);
-void launch_acct_bf16(const AcctArgs<float>& A, const AcctShape& sh, int n_accounts, cudaStream_t st);
-void launch_acct_fp32(const AcctArgs<float>& A, const AcctShape& sh, int n_accounts, cudaStream_t st);
+cudaError_t launch_acct_admm(const AcctArgs<T>& A, const AcctShape& sh, int n_accounts, cudaStream_t st);
+cudaError_t launch_acct_bf16(const AcctArgs<float>& A, const AcctShape& sh, int n_accounts, cudaStream_t st);
+cudaError_t launch_acct_fp32(const AcctArgs<float>& A, const AcctShape& sh, int n_accounts, cudaStream_t st);
 
 }  // namespace prism

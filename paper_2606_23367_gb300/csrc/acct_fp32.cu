@@ -3,8 +3,8 @@
 
 namespace prism {
 
-void launch_acct_fp32(const AcctArgs<float>& A, const AcctShape& sh, int n, cudaStream_t st) {
-    launch_acct_float<float>(A, sh, n, st);
+cudaError_t launch_acct_fp32(const AcctArgs<float>& A, const AcctShape& sh, int n, cudaStream_t st) {
+    return launch_acct_float<float>(A, sh, n, st);
 }
 
 }  // namespace prism

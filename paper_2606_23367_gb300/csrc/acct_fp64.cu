@@ -6,8 +6,6 @@ namespace prism {
 // ---------------------------------------------------------------------------
 // launch shapes
 // ---------------------------------------------------------------------------
-constexpr size_t ACCT_SMEM = 227 * 1024;
-
 static size_t acct_fixed(size_t t_bytes) {
     const size_t s = t_bytes == 8 ? sizeof(AcctShared<double>) : sizeof(AcctShared<float>);
     return (s + 15) / 16 * 16;
@@ -40,21 +38,19 @@ AcctShape acct_shape(int n, int K, int bytes_b, bool fac, bool pw) {
 }
 
 template <>
-void launch_acct_admm<float>(const AcctArgs<float>& A, const AcctShape& sh, int n, cudaStream_t st) {
-    if (A.B16p) launch_acct_bf16(A, sh, n, st);
-    else launch_acct_fp32(A, sh, n, st);
+cudaError_t launch_acct_admm<float>(const AcctArgs<float>& A, const AcctShape& sh, int n, cudaStream_t st) {
+    return A.B16p ? launch_acct_bf16(A, sh, n, st) : launch_acct_fp32(A, sh, n, st);
 }
 
 template <>
-void launch_acct_admm<double>(const AcctArgs<double>& A, const AcctShape& sh, int n, cudaStream_t st) {
+cudaError_t launch_acct_admm<double>(const AcctArgs<double>& A, const AcctShape& sh, int n, cudaStream_t st) {
     const bool gen = A.pw_idx || A.flo || A.tau;
     if (sh.E == 1) {
-        if (gen) launch_one<double, double, 1, 256, true, false>(A, sh, n, st);
-        else launch_one<double, double, 1, 256, false, false>(A, sh, n, st);
-    } else {
-        if (gen) launch_one<double, double, 2, 512, true, false>(A, sh, n, st);
-        else launch_one<double, double, 2, 512, false, false>(A, sh, n, st);
+        if (gen) return launch_one<double, double, 1, 256, true, false>(A, sh, n, st);
+        return launch_one<double, double, 1, 256, false, false>(A, sh, n, st);
     }
+    if (gen) return launch_one<double, double, 2, 512, true, false>(A, sh, n, st);
+    return launch_one<double, double, 2, 512, false, false>(A, sh, n, st);
 }
 
 }  // namespace prism

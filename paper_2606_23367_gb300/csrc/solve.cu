@@ -1232,15 +1232,15 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         if (o->time_budget_s > 0)                     // (FP64 iterations run through: checked between accounts)
             AF.budget_ns = (unsigned long long)(std::min(o->time_budget_s, 1e9) * 1e9) + 1;
     };
-    // the accounts' iterations in one launch
+    // the accounts' iterations in one launch (refused: the call fails before the polish is queued)
+    cudaError_t acct_err = cudaSuccess;
     auto run_acct = [&](int resume, double eps, int max_iter) {
         set_budget();
         AF.resume = AD.resume = resume;
         AF.eps = (float)eps; AD.eps = eps;
         AF.max_iter = AD.max_iter = max_iter;
         SC.prof.run(PRISM_K_BLOCK, 1, st, [&] {
-            if (fp64) launch_acct_admm(AD, shape, M, st);
-            else launch_acct_admm(AF, shape, M, st);
+            acct_err = fp64 ? launch_acct_admm(AD, shape, M, st) : launch_acct_admm(AF, shape, M, st);
         });
     };
     // A batched book with only a few accounts left to iterate goes on account-resident once their CTAs
@@ -1257,7 +1257,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         AF.max_iter = max_iter;
         AF.order = PK.order;
         set_budget();
-        SC.prof.run(PRISM_K_BLOCK, 1, st, [&] { launch_acct_admm(AF, again, (int)order_h.size(), st); });
+        SC.prof.run(PRISM_K_BLOCK, 1, st, [&] { acct_err = launch_acct_admm(AF, again, (int)order_h.size(), st); });
     };
     auto admm_loop = [&](int iter_budget, bool overlap) -> int {
         int done_iters = 0;
@@ -1370,6 +1370,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     if (D.fused && o->fold_products) { D.needP = needP_buf; D.fold = 1; }
     int total_iters = blockwise ? 0 : admm_loop(o->max_iter + check_every - cold, true);
     if (total_iters >= 0) total_iters += cold;
+    if (acct_err != cudaSuccess) { set_error(std::string("ADMM launch failed: ") + cudaGetErrorString(acct_err)); return PRISM_ERR_CUDA; }
     if (total_iters == -2) { set_error("tensor-core pipeline wait timed out (error flags " + std::to_string(SC.pinned[1]) + ")"); return PRISM_ERR_CUDA; }
     if (total_iters < 0) { set_error(std::string("ADMM loop failed: ") + cudaGetErrorString(cudaGetLastError())); return PRISM_ERR_CUDA; }
     SC.prof.run(PRISM_K_OTHER, 1, st, [&] { launch_mark_timeout(D, st); });   // accounts still iterating
@@ -1460,6 +1461,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
             more = admm_loop(D.max_iter, false);
             D = saved;
         }
+        if (acct_err != cudaSuccess) { set_error(std::string("ADMM launch failed: ") + cudaGetErrorString(acct_err)); return PRISM_ERR_CUDA; }
         if (more == -2) { set_error("tensor-core pipeline wait timed out"); return PRISM_ERR_CUDA; }
         if (more < 0) { set_error("ADMM retry failed"); return PRISM_ERR_CUDA; }
         total_iters += more;

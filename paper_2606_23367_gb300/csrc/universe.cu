@@ -343,7 +343,8 @@ static int create(const prism_universe_desc* desc, Universe& U) {
     IA.out[0] = U.d_Cinv32; IA.out[1] = U.d_Cinv16; IA.out[2] = U.d_CinvF32; IA.out[3] = U.d_CinvF16;
     IA.G_out[0] = U.d_G32; IA.G_out[1] = U.d_G16;
     const int smem = 2 * K * (K + 1) * (int)sizeof(double);
-    cudaFuncSetAttribute(k_cinv, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // (the limit belongs to the process: every thread sets the same one, whatever its K)
+    cudaFuncSetAttribute(k_cinv, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * KMAX * (KMAX + 1) * (int)sizeof(double));
     k_cinv<<<dim3(NRHO, 4), 256, smem, U.stream>>>(IA);
     int bad = 0;
     cudaError_t e = cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, U.stream);
