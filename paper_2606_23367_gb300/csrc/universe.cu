@@ -263,8 +263,7 @@ static int create(const prism_universe_desc* desc, Universe& U) {
     U.nseg = qseg[U.nq];
     cudaError_t se = cudaStreamCreateWithFlags(&U.stream, cudaStreamNonBlocking);
     if (se != cudaSuccess) { set_error(cudaGetErrorString(se)); return PRISM_ERR_CUDA; }
-    // One device block: what the host fills first (uploaded in one copy), then what the kernels fill,
-    // then their scratch. (27 allocations and 15 copies cost 0.5 ms here and their frees as much again.)
+    // One device block: what the host fills first (uploaded in one copy), then what the kernels fill. (27 allocations and 15 copies cost 0.5 ms here and their frees as much again.)
     std::vector<char> image;
     size_t off = 0;
     std::vector<std::pair<void**, size_t>> at;
@@ -308,16 +307,21 @@ static int create(const prism_universe_desc* desc, Universe& U) {
     place(&U.d_G16, (size_t)NRHO * K * K);
     place(&U.d_CinvF32, (size_t)NRHO * K * K);
     place(&U.d_CinvF16, (size_t)NRHO * K * K);
-    double *G = nullptr, *raw = nullptr;
+    // what only the setup needs: the Gram matrices, and B in the caller's order unless it is there already
     const bool here = on_device(desc->B, desc->device);
-    place(&G, 2 * (size_t)NRHO * K * K);
-    place(&raw, here ? 0 : (size_t)N * K);
-    if (cudaMalloc((void**)&U.d_block, off) != cudaSuccess) {
+    struct Scratch {
+        double* p = nullptr;
+        ~Scratch() { if (p) cudaFree(p); }
+    } scratch;
+    const size_t nG = 2 * (size_t)NRHO * K * K;
+    if (cudaMalloc((void**)&U.d_block, off) != cudaSuccess ||
+        cudaMalloc((void**)&scratch.p, (nG + (here ? 0 : (size_t)N * K)) * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         set_error("cudaMalloc (universe) failed");
         free_universe(U);
         return PRISM_ERR_ALLOCATION;
     }
+    double *const G = scratch.p, *const raw = scratch.p + nG;
     U.bytes = off;
     for (auto& q : at) *q.first = U.d_block + q.second;
     // (the default stream's copies order the upload behind what the caller queued there; they return

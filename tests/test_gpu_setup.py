@@ -75,3 +75,20 @@ def test_a_rejected_account_returns_zeros_beside_others():
     first = gpu_solve(uni, batch, precision=prism.PRISM_BATCHED_BF16)
     assert first["status"].tolist() == [prism.PRISM_CERTIFIED, prism.PRISM_NO_FEASIBLE_RETURN, prism.PRISM_CERTIFIED]
     assert not np.any(first["w"][sl])
+
+
+@pytest.mark.parametrize("device", [False, True])
+def test_a_universe_holds_its_arrays_and_no_scratch(device):
+    N, K = 100_000, 64
+    uni, _ = make_workload(1, N=N, K=K, M=1)
+    if device:
+        uni = _on_device(uni, ("B",))
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    h = prism.create_universe(uni)
+    held = before - torch.cuda.mem_get_info()[0]
+    h.close()
+    # B in FP64, FP32 and BF16, and padded and transposed copies of the last two; per asset some 40 bytes of the
+    # model and the order; per penalty six matrices in FP32; blocks of 2 MB
+    want = N * (8 * K + 2 * 4 * K + 4 * 2 * K + 40) + 33 * 6 * 4 * K * K
+    assert held <= want + (4 << 20), (held, want)
