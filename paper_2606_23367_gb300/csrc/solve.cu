@@ -1090,10 +1090,8 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         PRISM_CUDA_TRY(cudaMemcpyAsync(PK.order, order_h.data(), (size_t)M * 4, cudaMemcpyHostToDevice, st));
     }
     // ---- control init (see k_setup)
-    if (!acct) {
-        cudaMemsetAsync(D.v, 0, MN * 4, st);
-        if (D.stats) cudaMemsetAsync(D.stats, 0, 32, st);
-    }
+    if (!acct) cudaMemsetAsync(D.v, 0, MN * 4, st);
+    if (D.stats) cudaMemsetAsync(D.stats, 0, 32, st);
     SC.prof.run(PRISM_K_OTHER, acct ? 1 : 2, st, [&] {
         k_capacity<<<M, 256, 0, st>>>(S, N, Npad, U.d_sec_start, BD.lo, BD.up, BD.w0, BD.lof, BD.upf, BD.w0f,
                                       BD.band_lo, BD.band_hi, BD.tau, D.status, P.skip, D.active, P.W);

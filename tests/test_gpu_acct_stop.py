@@ -72,3 +72,18 @@ def test_a_tilt_that_cancels_mu_is_certified_on_exact_conditions(shift):
     assert np.mean(res["status"] == prism.PRISM_CERTIFIED) >= 0.5
     sure = np.repeat(res["status"] == prism.PRISM_CERTIFIED, np.diff(batch.offsets))
     assert float(np.max(np.abs(res["w"] - base["w"])[sure])) <= 1e-9
+
+
+def test_debug_counters_are_those_of_the_call(monkeypatch, capfd):
+    # on a handle whose last call counted the batched kernels' root evaluations
+    monkeypatch.setenv("PRISM_DEBUG_STATS", "1")
+    uni, batch = make_workload(1, N=900, K=16, M=6)
+    h = prism.create_universe(uni)
+    try:
+        for opts in (dict(chains=1), {}):
+            capfd.readouterr()
+            prism.solve(h, batch, precision=prism.PRISM_BATCHED_BF16, **opts)
+            err = capfd.readouterr().err
+            assert ("prox account-calls 0," in err) == (not opts), err
+    finally:
+        h.close()
