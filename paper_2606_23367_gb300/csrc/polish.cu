@@ -1424,7 +1424,8 @@ __global__ void k_adjoint_flags(PolDev P, uint8_t* flags) {
     const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (size_t)P.M * P.Npad) return;
     const int p = int(e % P.Npad);
-    if (p >= P.N) { flags[e] = 0; return; }
+    // (a rejected account was never classified: its state codes are whatever the memory held)
+    if (p >= P.N || (P.skip && P.skip[e / P.Npad])) { flags[e] = 0; return; }
     Pieces pc;
     entry_pieces(P, e, pc);
     const int code = P.st[e];

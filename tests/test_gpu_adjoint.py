@@ -179,3 +179,22 @@ def test_autograd_function_matches_the_c_abi(device):
     assert np.allclose(c(B.grad), ref["dB"], rtol=1e-12, atol=1e-12)
     assert np.allclose(c(d.grad), ref["dd"], rtol=1e-12, atol=1e-12)
     assert np.allclose(c(w0.grad), ref["dw0"], rtol=1e-12, atol=1e-12)
+
+
+def test_a_rejected_account_has_no_gradient():
+    # it is never classified, so that its entries have no state codes to read
+    uni, batch = make_workload(4, N=600, K=16, M=3)
+    sl = batch.account_slice(1)
+    batch.upper[sl] = 1e-4                             # capacity far below the budget
+    g = np.random.default_rng(0).normal(size=len(batch.w0))
+
+    def gradients(b, g):
+        res = prism.solve(prism.create_universe(uni), b, keep_for_backward=1)
+        return res["status"].tolist(), prism.prism_solve_batch_backward(res["state"], g)
+
+    status, got = gradients(batch, g)
+    assert status == [prism.PRISM_CERTIFIED, prism.PRISM_NO_FEASIBLE_RETURN, prism.PRISM_CERTIFIED]
+    assert not np.any(got["dw0"][sl])
+    _, ref = gradients(batch.subset([0, 2]), np.concatenate([g[batch.account_slice(a)] for a in (0, 2)]))
+    for k in ("dmu", "dB", "dd"):
+        assert_close(got[k], ref[k], k)
