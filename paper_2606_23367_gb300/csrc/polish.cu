@@ -847,12 +847,6 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) k_polish(PolDev P, int 
                 }
             }
             sh.nc = nc;
-            // A cap that depends on the budget (every free weight on one side of its holding) keeps the
-            // iterations' multiplier: the budget's takes up the difference on the free weights, while
-            // with theta = 0 nearly every held name would seem to want to move
-            if (P.theta_hint)
-                for (int r = 1; r < m; ++r)
-                    if (!sh.used[r] && sh.rows[r] == S) sh.lam[r] = fmax(double(P.theta_hint[a]), 0.0);
             sh.fail = (nc == 0);
         }
         __syncthreads();

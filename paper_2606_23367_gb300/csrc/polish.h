@@ -48,7 +48,6 @@ struct PolDev {
     const float* eta_hi_f = nullptr;    // M x S
     const float* eta_lo_f = nullptr;
     const float* theta_f = nullptr;     // M
-    const float* theta_hint = nullptr;  // M, or null: the cap multiplier of the iterations
     int* skip = nullptr;                // M: 1 = leave this account alone
     const int* sel = nullptr;           // M: when set, only the accounts with sel[a] == gen
     int gen = 0;

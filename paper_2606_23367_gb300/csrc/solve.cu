@@ -227,6 +227,17 @@ __global__ void k_setup(SetupArgs A) {
     }
 }
 
+// The accounts that iterate on (active) begin again: what a first pass of the iterations starts from.
+__global__ void k_restart(int M, int S, Dev D, int rho_idx) {
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < (int64_t)M * S && D.active[e / S]) D.eta_hi[e] = D.eta_lo[e] = __int_as_float(-1);
+    if (e < M && D.active[e]) {
+        D.rho_idx[e] = rho_idx;
+        D.iters[e] = 0;
+        D.nu[e] = D.theta[e] = 0.f;
+    }
+}
+
 // The number of accounts that the polish left for another pass of the iterations.
 __global__ void k_unsettled(int M, const int* skip, const int* done, const int* status, int* n) {
     int c = 0;
@@ -910,11 +921,12 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     flush();
     if (nnz > 0) SC.prof.run(PRISM_K_PACK, 1, st, [&] { k_pack<<<(unsigned)cdiv64(nnz, 256), 256, 0, st>>>(PA); });
     // bands, caps, factor bounds and the accounts' state
+    const int j0 = (int)std::lround(RHO_PER_DECADE * std::log10(std::max(o->rho0, 1e-12) / RHO_MIN));
+    const int rho_idx0 = std::max(0, std::min(NRHO - 1, j0));
     {
         SetupArgs SA = {};
         SA.M = M; SA.S = S; SA.K = K;
-        int j0 = (int)std::lround(RHO_PER_DECADE * std::log10(std::max(o->rho0, 1e-12) / RHO_MIN));
-        SA.rho_idx = std::max(0, std::min(NRHO - 1, j0));
+        SA.rho_idx = rho_idx0;
         SA.n_ctr = 2 * SolveCache::MAXCH;
         SA.band_lo = (const double*)stage_in(b->band_lo, BD.band_lo, (size_t)M * S * 8);
         SA.band_hi = (const double*)stage_in(b->band_hi, BD.band_hi, (size_t)M * S * 8);
@@ -1044,7 +1056,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     P.band_lo = BD.band_lo; P.band_hi = BD.band_hi; P.tau = BD.tau;
     if (BD.has_fac) { P.flo = BD.flo; P.fhi = BD.fhi; P.sflag = D.sflag; }
     else P.wfac = nullptr;
-    P.z = D.z; P.nu_f = D.nu; P.eta_hi_f = D.eta_hi; P.eta_lo_f = D.eta_lo; P.theta_f = D.theta; P.theta_hint = D.theta;
+    P.z = D.z; P.nu_f = D.nu; P.eta_hi_f = D.eta_hi; P.eta_lo_f = D.eta_lo; P.theta_f = D.theta;
     P.FMAX = FMAX;
     P.status = D.status;
     P.tol_dual = 1e-11; P.tol_primal = 1e-12;
@@ -1197,11 +1209,6 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
             A.rho_idx = D.rho_idx; A.iters = D.iters; A.active = D.active; A.status = D.status;
             if (BD.has_fac) A.sflag = D.sflag;
             A.t0 = t0_dev;
-            // With lots or a cap the polish can lose its way from a start a few places off, and one such
-            // account costs it eight rounds on hundreds of free entries: 8-11 ms of a 200 x 1,924 book
-            // against 0.6 when every account first keeps its places for 12 iterations (ADMM 1.6 -> 2.2
-            // ms). Books without them gain nothing (100 x 5,000 x 48: 1.3 -> 2.3 against 0.67 -> 0.47).
-            A.settle = (has_lots || BD.has_cap) ? 12 : 0;
             A.alpha = o->alpha; A.eps = o->eps_admm;
             A.max_iter = o->max_iter; A.min_iter = o->min_iter; A.adapt_every = D.adapt_every;
         };
@@ -1230,10 +1237,18 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         if (o->time_budget_s > 0)                     // (FP64 iterations run through: checked between accounts)
             AF.budget_ns = (unsigned long long)(std::min(o->time_budget_s, 1e9) * 1e9) + 1;
     };
+    // With lots or a cap the polish can lose its way from a start a few places off, and one such account
+    // costs it eight rounds on hundreds of free entries: 8-11 ms of a 200 x 1,924 book against 0.6 when every
+    // account first keeps its places for 12 iterations (ADMM 1.6 -> 2.2 ms). Books without them gain
+    // nothing (100 x 5,000 x 48: 1.3 -> 2.3 against 0.67 -> 0.47). The few accounts that the polish leaves
+    // all the same begin again and take the batched kernels' passes, without that wait: which accounts
+    // certify is theirs (3 of 50,000 certify from there and not from the places that they kept).
+    const int settle = (acct && (has_lots || BD.has_cap)) ? 12 : 0;
     // the accounts' iterations in one launch (refused: the call fails before the polish is queued)
     cudaError_t acct_err = cudaSuccess;
-    auto run_acct = [&](int resume, double eps, int max_iter) {
+    auto run_acct = [&](int resume, double eps, int max_iter, int wait) {
         set_budget();
+        AF.settle = AD.settle = wait;
         AF.resume = AD.resume = resume;
         AF.eps = (float)eps; AD.eps = eps;
         AF.max_iter = AD.max_iter = max_iter;
@@ -1330,7 +1345,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
     const bool blockwise = acct || fp64 || packed;   // every iteration inside a per-account kernel
     const int cold = (D.stream_prox && !blockwise) ? std::min(std::max(0, o->stream_after), o->max_iter) : 0;
     if (acct) {
-        run_acct(0, o->eps_admm, o->max_iter);
+        run_acct(0, o->eps_admm, o->max_iter, settle);
     } else if (fp64) {
         // PLAIN_FP64: every iteration of the account in one FP64 launch (block_admm.cu)
         P64.resume = 0;
@@ -1382,7 +1397,8 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
                      h[0] ? double(h[1]) / h[0] : 0.0, h[0] ? double(h[2]) / h[0] : 0.0,
                      h[0] ? double(h[3]) / h[0] : 0.0);
     }
-    // ---- polish, with up to two returns to the iterations at a tighter target
+    // ---- polish, with up to two returns to the iterations at a tighter target (after a new start of
+    // accounts that had been waiting for their places)
     // polish rounds until no account needs another (checked after each round)
     int n_rounds_run = 0, n_retried = 0;
     // all active-set rounds of every account in one launch; each block stops when settled (one
@@ -1405,7 +1421,7 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         SC.prof.run(PRISM_K_OTHER, 1, st, [&] { launch_classify(P, st); });
         if (polish_rounds(false, M) < 0) { set_error("polish failed"); return PRISM_ERR_CUDA; }
     }
-    for (int retry = 0; retry < 2; ++retry) {
+    for (int retry = settle ? -1 : 0; retry < 2; ++retry) {   // (-1: they begin again, see settle)
         SC.prof.run(PRISM_K_OTHER, 1, st, [&] { k_unsettled<<<1, 1024, 0, st>>>(M, P.skip, P.done, D.status, err + 3); });
         PRISM_CUDA_TRY(cudaMemcpyAsync(SC.pinned + 8, err + 3, 4, cudaMemcpyDeviceToHost, st));
         PRISM_CUDA_TRY(cudaStreamSynchronize(st));
@@ -1435,8 +1451,11 @@ static int solve_core(prism_universe* uh, const prism_batch* b, const prism_solv
         PRISM_CUDA_TRY(cudaStreamSynchronize(st));
         int more = 0;
         const int sent_back = n_retry;
-        if (acct) {
-            run_acct(1, o->eps_admm * (retry == 0 ? 0.1 : 0.01), o->max_iter * (retry + 2));
+        if (retry < 0) {
+            SC.prof.run(PRISM_K_OTHER, 1, st, [&] { k_restart<<<(unsigned)cdiv64((int64_t)M * S, 256), 256, 0, st>>>(M, S, D, rho_idx0); });
+            run_acct(0, o->eps_admm, o->max_iter, 0);
+        } else if (acct) {
+            run_acct(1, o->eps_admm * (retry == 0 ? 0.1 : 0.01), o->max_iter * (retry + 2), 0);
         } else if (few_fit(n_retry)) {
             run_few(act.data(), o->eps_admm * (retry == 0 ? 0.1 : 0.01), o->max_iter * (retry + 2));
         } else if (fp64) {

@@ -92,3 +92,17 @@ def test_fp64_iterations_are_those_of_the_blocks(seed):
     assert int(np.max(np.abs(new["iters"] - old["iters"]))) <= 1
     for k in ("w", "nu", "lambda_band"):
         assert float(np.max(np.abs(new[k] - old[k]))) <= 1e-11, k
+
+
+@pytest.mark.parametrize("seed,N,K,M", [(1160, 492, 39, 162), (1023, 674, 21, 19), (37, 1924, 48, 200)])
+def test_lots_and_a_cap_certify_the_same_accounts(seed, N, K, M):
+    # books with an account that the polish leaves at first: it certifies where the batched kernels' does, and
+    # where it does not, its last polish started from the same iterate and left the same multipliers
+    uni, batch = make_workload(3, seed=seed, N=N, K=K, M=M)
+    new = gpu_solve(uni, batch, precision=prism.PRISM_BATCHED_BF16)
+    old = gpu_solve(uni, batch, precision=prism.PRISM_BATCHED_BF16, chains=1)
+    sure = old["status"] == prism.PRISM_CERTIFIED
+    assert new["kernel_launches"][BLOCK] > 0 and np.array_equal(new["status"] == prism.PRISM_CERTIFIED, sure)
+    for k in ("nu", "lambda_band", "theta"):
+        assert float(np.max(np.abs(new[k] - old[k]))) <= 1e-11, k
+    assert float(np.max(np.abs(new["w"] - old["w"])[np.repeat(sure, np.diff(batch.offsets))])) <= 1e-11
