@@ -226,7 +226,9 @@ void prism_default_opts(prism_solve_opts* o);
 typedef struct {
     double*  w;             /* ragged weights, same layout as prism_batch (required) */
     double*  nu;            /* M budget multipliers, or NULL */
-    double*  lambda_band;   /* M x S band multipliers, or NULL */
+    double*  lambda_band;   /* M x S band multipliers, or NULL. Not unique on an edge that the bounds of
+                               the sector's own entries imply (a floor of 0 on a sector sold out): then
+                               0 or the bounds' multiplier, the routes of a book alike */
     double*  theta;         /* M cap multipliers, or NULL */
     int32_t* status;        /* M per-account status (required) */
     int32_t* iters;         /* M ADMM iterations used, or NULL */
